@@ -56,7 +56,7 @@ TUNING = {"blocks_per_sm": 4}
 # checks these figures against the counts.
 FLOP_PER_TET = 222.0
 FLOP_PER_BBOX_CELL = 29.0
-FLOP_PER_RUN = 2000.0
+FLOP_PER_RUN = 1310.0
 SM_COUNT_GB300 = 152
 SM_MAX_MHZ_GB300 = 2070.0  # the part's maximum SM clock
 FP32_LANES_PER_SM = 128

@@ -32,6 +32,37 @@ namespace pse {
 // plane; the line crosses the face inside the tetrahedron's bounding box, so o_c stays
 // within a few cells of the origin.
 // ---------------------------------------------------------------------------
+// The edge list of one clipped face polygon: up to 7 directed edges a -> b.  A float slot is one
+// float4 (a.xyz, b.x) and one float2 (b.yz) on the device, so that a lane reads it with two
+// loads; any other scalar type (and the host) keeps three two-scalar rows per slot.  Slots of
+// neighbouring lanes are adjacent (a stride of 32 lanes), so accesses have no bank conflicts.
+template <class T>
+struct EdgeSlots {
+    slot2_t<T> *e;
+    PSE_HD void store(int k, const P3<T> &a, const P3<T> &b) const { slot_store<T>(e, k, a, b); }
+    PSE_HD void load(int k, P3<T> &a, P3<T> &b) const { slot_load<T>(e, k, a, b); }
+};
+#ifdef __CUDACC__
+// the float slots of one lane of a warp: h points into a [7][32] float4 block, l into a
+// [7][32] float2 block
+struct EdgeSlots4 {
+    float4 *h;
+    float2 *l;
+    __device__ __forceinline__ void store(int k, const P3<float> &a, const P3<float> &b) const
+    {
+        h[32 * k] = make_float4(a.x, a.y, a.z, b.x);
+        l[32 * k] = make_float2(b.y, b.z);
+    }
+    __device__ __forceinline__ void load(int k, P3<float> &a, P3<float> &b) const
+    {
+        const float4 u = h[32 * k];
+        const float2 v = l[32 * k];
+        a = mk<float>(u.x, u.y, u.z);
+        b = mk<float>(u.w, v.x, v.y);
+    }
+};
+#endif
+
 template <class T>
 struct FaceSums {
     T m6;          // 6 ∫ (z - l) over the clipped face polygon (signed by orientation)
@@ -40,77 +71,193 @@ struct FaceSums {
     T zmin, zmax;  // z range of the polygon's vertices
 };
 
-// y slab pass of the column clip: slab_pass<1> on the slots in E, and the face sums of the
-// clipped polygon (its surviving edges and the two new ones on the y planes).
-template <class T>
-PSE_HD void yslab_sums(slot2_t<T> *E, T lo, T hi, T tol, const P3<T> &o, T fo, T l0, T lx, T ly, FaceSums<T> &I)
+// 1 / x for the slab passes: the device's approximate reciprocal, whose result is only used
+// clamped to an edge.  A difference of 0 (or one too small for it: flushed) gives an infinity,
+// and the products with it 0, 1 or, clamped, 0 for NaN: a point of the edge all the same.
+PSE_HD float slab_rcp(float x)
 {
-    constexpr int ne = 5;
-    const P3<T> z0 = mk<T>(T(0), T(0), T(0));
-    P3<T> xl = z0, nl = z0, xh = z0, nh = z0;
+#ifdef __CUDA_ARCH__
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+#else
+    return 1.f / x;
+#endif
+}
+template <class T>
+PSE_HD T slab_rcp(T x)
+{
+    return fdiv(T(1), x);
+}
+
+// The sums below are written with explicit fused multiply-adds and separately rounded products,
+// so that every kernel forms them alike, however the compiler would fuse them: a fan triangle's
+// term and the integral of l over it (see fan_mid).
+template <class T>
+PSE_HD T fan_height(const P3<T> &a, const P3<T> &b, T fo, T l0, T lx, T ly)
+{
+    const T fa = a.z - fmaT(lx, a.x, fmaT(ly, a.y, l0));
+    const T fb = b.z - fmaT(lx, b.x, fmaT(ly, b.y, l0));
+    return fo + fa + fb;
+}
+template <class T>
+PSE_HD T plane_sum(const P3<T> &a, const P3<T> &b, T l0, T lx, T ly)
+{
+    return fmaT(T(3), l0, fmaT(lx, a.x + b.x, mul_rn(ly, a.y + b.y)));
+}
+
+// x slab pass of the column clip: the triangle (a, b, c) clipped against lo <= x < hi, its
+// surviving edges stored in order (the triangle's, then the new ones on lo and on hi); returns
+// their number (0 to 5).  An edge is cut at its own parameters for the two planes, each end by
+// the plane it lies beyond; an edge beyond one plane at both ends is left out (it would add
+// exactly 0 to every sum).  The vertices' sides are found once per vertex.
+template <class T, class Slots>
+PSE_HD int xslab_triangle(const P3<T> &a, const P3<T> &b, const P3<T> &c, T lo, T hi, T tol, const Slots &E)
+{
+    const P3<T> p[3] = {a, b, c};
+    const T lt = lo - tol, ht = hi - tol;
+    bool below[3], above[3];
+    T cx[3];  // x of the vertex moved into the slab
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        below[i] = p[i].x < lt;
+        above[i] = p[i].x >= ht;
+        cx[i] = below[i] ? lo : (above[i] ? hi : p[i].x);
+    }
+    // exit and entry points on the two planes (a triangle crosses each at most once each way)
+    T xly = T(0), xlz = T(0), nly = T(0), nlz = T(0), xhy = T(0), xhz = T(0), nhy = T(0), nhz = T(0);
+    int n = 0;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const int j = i == 2 ? 0 : i + 1;
+        const T inv = slab_rcp(p[j].x - p[i].x);
+        const T ta = sat01(((below[i] ? lo : hi) - p[i].x) * inv), tb = sat01(((below[j] ? lo : hi) - p[i].x) * inv);
+        const T dy = p[j].y - p[i].y, dz = p[j].z - p[i].z;
+        const bool ina = !below[i] && !above[i], inb = !below[j] && !above[j];
+        const T ay = ina ? p[i].y : fmaT(ta, dy, p[i].y), az = ina ? p[i].z : fmaT(ta, dz, p[i].z);
+        const T by = inb ? p[j].y : fmaT(tb, dy, p[i].y), bz = inb ? p[j].z : fmaT(tb, dz, p[i].z);
+        const bool xl = !below[i] && below[j], nl = below[i] && !below[j];
+        const bool xh = !above[i] && above[j], nh = above[i] && !above[j];
+        xly = xl ? by : xly;
+        xlz = xl ? bz : xlz;
+        nly = nl ? ay : nly;
+        nlz = nl ? az : nlz;
+        xhy = xh ? by : xhy;
+        xhz = xh ? bz : xhz;
+        nhy = nh ? ay : nhy;
+        nhz = nh ? az : nhz;
+        if (!(below[i] && below[j]) && !(above[i] && above[j])) {
+            E.store(n, mk<T>(cx[i], ay, az), mk<T>(cx[j], by, bz));
+            ++n;
+        }
+    }
+    if ((below[0] || below[1] || below[2]) && !(below[0] && below[1] && below[2])) {
+        E.store(n, mk<T>(lo, xly, xlz), mk<T>(lo, nly, nlz));
+        ++n;
+    }
+    if ((above[0] || above[1] || above[2]) && !(above[0] && above[1] && above[2])) {
+        E.store(n, mk<T>(hi, xhy, xhz), mk<T>(hi, nhy, nhz));
+        ++n;
+    }
+    return n;
+}
+
+// y slab pass of the column clip on the n edges in E, and the face sums of the clipped polygon
+// (its surviving edges and the two new ones on the y planes).  The surviving edges of nonzero
+// length are stored back in order, the new ones after them; returns their number (0 to 7).
+template <class T, class Slots>
+PSE_HD int yslab_sums(const Slots &E, int n, T lo, T hi, T tol, const P3<T> &o, T fo, T l0, T lx, T ly, FaceSums<T> &I)
+{
+    const T lt = lo - tol, ht = hi - tol;
+    P3<T> xl = mk<T>(T(0), lo, T(0)), nl = xl, xh = mk<T>(T(0), hi, T(0)), nh = xh;
+    bool cl = false, ch = false;  // the polygon crosses lo / hi
     T m6 = T(0), x2 = T(0), y6 = T(0);
     T zmn = T(1e30), zmx = T(-1e30);  // an empty polygon keeps this range
+    int m = 0;
 #pragma unroll 1
-    for (int k = 0; k < ne; ++k) {
+    for (int k = 0; k < n; ++k) {
         P3<T> ea, eb;
-        slot_load<T>(E, k, ea, eb);
-        const bool a_lo = ea.y < lo - tol, b_lo = eb.y < lo - tol;
-        const bool a_hi = ea.y >= hi - tol, b_hi = eb.y >= hi - tol;
-        const T inv = fdiv(T(1), eb.y - ea.y);
-        const P3<T> pa = at_plane(ea, eb, sat01((lo - ea.y) * inv), 1, lo);
-        const P3<T> ph = at_plane(ea, eb, sat01((hi - ea.y) * inv), 1, hi);
-        const P3<T> na = a_lo ? pa : (a_hi ? ph : ea);
-        const P3<T> nb = b_lo ? pa : (b_hi ? ph : eb);
-        slot_store<T>(E, k, na, nb);
-        xl = (!a_lo && b_lo) ? pa : xl;
-        nl = (a_lo && !b_lo) ? pa : nl;
-        xh = (!a_hi && b_hi) ? ph : xh;
-        nh = (a_hi && !b_hi) ? ph : nh;
+        E.load(k, ea, eb);
+        const bool a_lo = ea.y < lt, b_lo = eb.y < lt;
+        const bool a_hi = ea.y >= ht, b_hi = eb.y >= ht;
+        const T inv = slab_rcp(eb.y - ea.y);
+        const T pa = a_lo ? lo : hi, pb = b_lo ? lo : hi;  // the plane an end outside is cut by
+        const T ta = sat01((pa - ea.y) * inv), tb = sat01((pb - ea.y) * inv);
+        const T dx = eb.x - ea.x, dz = eb.z - ea.z;
+        const bool ina = !a_lo && !a_hi, inb = !b_lo && !b_hi;
+        const P3<T> na = mk<T>(ina ? ea.x : fmaT(ta, dx, ea.x), ina ? ea.y : pa, ina ? ea.z : fmaT(ta, dz, ea.z));
+        const P3<T> nb = mk<T>(inb ? eb.x : fmaT(tb, dx, ea.x), inb ? eb.y : pb, inb ? eb.z : fmaT(tb, dz, ea.z));
+        const bool oxl = !a_lo && b_lo, onl = a_lo && !b_lo, oxh = !a_hi && b_hi, onh = a_hi && !b_hi;
+        xl.x = oxl ? nb.x : xl.x;
+        xl.z = oxl ? nb.z : xl.z;
+        nl.x = onl ? na.x : nl.x;
+        nl.z = onl ? na.z : nl.z;
+        xh.x = oxh ? nb.x : xh.x;
+        xh.z = oxh ? nb.z : xh.z;
+        nh.x = onh ? na.x : nh.x;
+        nh.z = onh ? na.z : nh.z;
+        cl = cl || oxl;
+        ch = ch || oxh;
         // a dropped edge has zero length: it adds nothing to the sums
         const T cr = cross_xy(na, nb);
-        m6 += fan_mid(na, nb, o, fo, l0, lx, ly);
+        m6 = fmaT(cross_xy(sub(na, o), sub(nb, o)), fan_height(na, nb, fo, l0, lx, ly), m6);
         x2 += cr;
-        y6 += cr * fmaT(T(3), l0, fmaT(lx, na.x + nb.x, ly * (na.y + nb.y)));
+        y6 = fmaT(cr, plane_sum(na, nb, l0, lx, ly), y6);
         // z range over edges of nonzero length (dropped edges carry no vertex of the polygon)
         const bool live = na.x != nb.x || na.y != nb.y || na.z != nb.z;
-        zmn = live ? fmin(zmn, fmin(na.z, nb.z)) : zmn;
-        zmx = live ? fmax(zmx, fmax(na.z, nb.z)) : zmx;
+        if (live) {
+            zmn = fmin(zmn, fmin(na.z, nb.z));
+            zmx = fmax(zmx, fmax(na.z, nb.z));
+            E.store(m, na, nb);
+            ++m;
+        }
     }
-    slot_store<T>(E, ne, xl, nl);
-    slot_store<T>(E, ne + 1, xh, nh);
     // the new edges join points that already bound surviving edges: they change no z range
     {
         const T c1 = cross_xy(xl, nl), c2 = cross_xy(xh, nh);
-        m6 += fan_mid(xl, nl, o, fo, l0, lx, ly) + fan_mid(xh, nh, o, fo, l0, lx, ly);
+        m6 += fmaT(cross_xy(sub(xh, o), sub(nh, o)), fan_height(xh, nh, fo, l0, lx, ly),
+                   mul_rn(cross_xy(sub(xl, o), sub(nl, o)), fan_height(xl, nl, fo, l0, lx, ly)));
         x2 += c1 + c2;
-        y6 += c1 * fmaT(T(3), l0, fmaT(lx, xl.x + nl.x, ly * (xl.y + nl.y))) +
-              c2 * fmaT(T(3), l0, fmaT(lx, xh.x + nh.x, ly * (xh.y + nh.y)));
+        y6 += fmaT(c2, plane_sum(xh, nh, l0, lx, ly), mul_rn(c1, plane_sum(xl, nl, l0, lx, ly)));
+    }
+    if (cl) {
+        E.store(m, xl, nl);
+        ++m;
+    }
+    if (ch) {
+        E.store(m, xh, nh);
+        ++m;
     }
     I.m6 = m6;
     I.x2 = x2;
     I.y6 = y6;
     I.zmin = zmn;
     I.zmax = zmx;
+    return m;
 }
 
-// 6 ∫ (z - c)_+ over the polygon in the 7 slots of E: fan from (ox, oy), a point of the face
-// plane at height c, over the parts of the edges above c.
-template <class T>
-PSE_HD T level_fan(const slot2_t<T> *E, T c, T ox, T oy)
+// 6 ∫ (z - c)_+ over the polygon of the n edges in E: fan from s (nx, ny), a point of the face
+// plane at height c, over the parts of the edges above c.  FUSED: the offsets from that point
+// are formed with one rounding (the octree kernels) instead of from its rounded coordinates (the
+// uniform ones); the two differ in the last bit only, and each kernel keeps to one of them.
+template <bool FUSED, class T, class Slots>
+PSE_HD T level_fan(const Slots &E, int n, T c, T s, T nx, T ny)
 {
+    const T ox = mul_rn(s, nx), oy = mul_rn(s, ny);
     T g = T(0);
 #pragma unroll 1
-    for (int k = 0; k < 7; ++k) {
+    for (int k = 0; k < n; ++k) {
         P3<T> ea, eb;
-        slot_load<T>(E, k, ea, eb);
+        E.load(k, ea, eb);
         const bool a_up = ea.z > c, b_up = eb.z > c;
         const T t = (c - ea.z) * fdiv(T(1), eb.z - ea.z);
         const T px = fmaT(t, eb.x - ea.x, ea.x), py = fmaT(t, eb.y - ea.y, ea.y);
-        const T ax = (a_up ? ea.x : px) - ox, ay = (a_up ? ea.y : py) - oy;
-        const T bx = (b_up ? eb.x : px) - ox, by = (b_up ? eb.y : py) - oy;
+        const T ux = a_up ? ea.x : px, uy = a_up ? ea.y : py, vx = b_up ? eb.x : px, vy = b_up ? eb.y : py;
+        const T ax = FUSED ? fmaT(-s, nx, ux) : ux - ox, ay = FUSED ? fmaT(-s, ny, uy) : uy - oy;
+        const T bx = FUSED ? fmaT(-s, nx, vx) : vx - ox, by = FUSED ? fmaT(-s, ny, vy) : vy - oy;
         const T fa = a_up ? ea.z - c : T(0), fb = b_up ? eb.z - c : T(0);
         const T cr = mul_rn(ax, by) - mul_rn(ay, bx);
-        g += (a_up || b_up) ? cr * (fa + fb) : T(0);
+        g += (a_up || b_up) ? mul_rn(cr, fa + fb) : T(0);
     }
     return g;
 }
@@ -146,8 +293,8 @@ PSE_HD RunFrame<T> run_frame(const Src &src, T lx, T ly, int K, bool lo_open)
     F.qy = floor(fmin(fmax(cy, T(0)), T(1)) * T(256) + T(0.5)) * T(1.0 / 256);
     F.qz = floor(fmin(fmax(cz, T(0)), kf) * T(256) + T(0.5)) * T(1.0 / 256);
     const T xc = T(0.5) - F.qx, yc = T(0.5) - F.qy;
-    const T lc = fmin(fmax((cz - F.qz) + lx * (xc - (cx - F.qx)) + ly * (yc - (cy - F.qy)), -F.qz), kf - F.qz);
-    F.l0 = lc - lx * xc - ly * yc;
+    const T at = fmaT(ly, yc - (cy - F.qy), fmaT(lx, xc - (cx - F.qx), cz - F.qz));
+    F.l0 = fmaT(-ly, yc, fmaT(-lx, xc, fmin(fmax(at, -F.qz), kf - F.qz)));
     F.lx = lx;
     F.ly = ly;
     F.K = K;
@@ -155,22 +302,19 @@ PSE_HD RunFrame<T> run_frame(const Src &src, T lx, T ly, int K, bool lo_open)
     return F;
 }
 
-// Whether face f can reach the run's column (its projection's bounding box meets the column
-// and it is not vertical).
-template <class T, class Src>
-PSE_HD bool face_meets_column(const Src &src, int f, const RunFrame<T> &F)
+// Whether the face (a, b, c; local frame, normal z component nz) can reach the run's column: its
+// projection's bounding box meets the column and it is not vertical.
+template <class T>
+PSE_HD bool face_meets_column(const P3<T> &a, const P3<T> &b, const P3<T> &c, T nz, const RunFrame<T> &F)
 {
-    int ia, ib, ic;
-    face_vertices(f, ia, ib, ic);
-    const P3<T> a = src.vtx(ia), b = src.vtx(ib), c = src.vtx(ic);
-    const T mnx = fmin(a.x, fmin(b.x, c.x)) - F.qx, mxx = fmax(a.x, fmax(b.x, c.x)) - F.qx;
-    const T mny = fmin(a.y, fmin(b.y, c.y)) - F.qy, mxy = fmax(a.y, fmax(b.y, c.y)) - F.qy;
+    const T mnx = fmin(a.x, fmin(b.x, c.x)), mxx = fmax(a.x, fmax(b.x, c.x));
+    const T mny = fmin(a.y, fmin(b.y, c.y)), mxy = fmax(a.y, fmax(b.y, c.y));
     if (mxx < -F.qx || mnx >= T(1) - F.qx || mxy < -F.qy || mny >= T(1) - F.qy) return false;
-    return src.nrm(f).z != T(0);
+    return nz != T(0);
 }
 
-// One face of a run: the x and y slab passes (the clipped polygon is left in the 7 slots of
-// E), then 6 x its term of B(c_j) for the levels j0 .. K by the closed forms (a level the
+// One face of a run: the x and y slab passes (the clipped polygon is left in the first n slots
+// of E), then 6 x its term of B(c_j) for the levels j0 .. K by the closed forms (a level the
 // face straddles gets the "below" form m6; the fan of its part above the level is subtracted
 // afterwards, see level_fan), its z range, its moment, and the straddled levels jlo .. jhi
 // (empty when jlo > jhi) with the plane data their fans need.
@@ -178,35 +322,44 @@ template <int KW, class T>
 struct FaceRun {
     T k6[KW + 1];
     T zmin, zmax, m6;
-    int jlo, jhi;
+    int jlo, jhi, n;
     T nx, ny, nz, ef;  // face plane n . x = ef in the local frame
 };
 
-template <int KW, class T, class Src>
-PSE_HD void face_run(const Src &src, int f, const RunFrame<T> &F, slot2_t<T> *E, FaceRun<KW, T> &R)
+// a face that adds nothing to the run
+template <int KW, class T>
+PSE_HD void face_none(FaceRun<KW, T> &R)
 {
-    int ia, ib, ic;
-    face_vertices(f, ia, ib, ic);
-    const P3<T> q = mk<T>(F.qx, F.qy, F.qz);
-    const P3<T> a = sub(src.vtx(ia), q), b = sub(src.vtx(ib), q), c = sub(src.vtx(ic), q);
-    const P3<T> nf = src.nrm(f);
+#pragma unroll
+    for (int j = 0; j <= KW; ++j) R.k6[j] = T(0);
+    R.zmin = T(1e30);
+    R.zmax = T(-1e30);
+    R.m6 = T(0);
+    R.jlo = 0;
+    R.jhi = -1;
+    R.n = 0;
+    R.nx = R.ny = R.nz = R.ef = T(0);
+}
+
+// (a, b, c): the face's vertices in the local frame, outward order; nf: its normal.
+template <int KW, class T, class Slots>
+PSE_HD void face_run(const P3<T> &a, const P3<T> &b, const P3<T> &c, const P3<T> &nf, const RunFrame<T> &F,
+                     const Slots &E, FaceRun<KW, T> &R)
+{
     const T mnx = fmin(a.x, fmin(b.x, c.x)), mxx = fmax(a.x, fmax(b.x, c.x));
     const T mny = fmin(a.y, fmin(b.y, c.y)), mxy = fmax(a.y, fmax(b.y, c.y));
     const T mnz = fmin(a.z, fmin(b.z, c.z)), mxz = fmax(a.z, fmax(b.z, c.z));
     const T cmag = fmax(T(1), fmax(fmax(fmax(fabs(mnx), fabs(mxx)), fmax(fabs(mny), fabs(mxy))),
                                    fmax(fabs(mnz), fabs(mxz))));
     const T tol = T(8) * roundoff<T>() * cmag;
-    const T ef = dot(nf, a);
-    const T sc = fdiv(ef, dot(nf, nf));
-    const P3<T> o = mk<T>(sc * nf.x, sc * nf.y, sc * nf.z);
-    const T fo = o.z - fmaT(F.lx, o.x, fmaT(F.ly, o.y, F.l0));
+    const T ef = fmaT(nf.z, a.z, fmaT(nf.x, a.x, mul_rn(nf.y, a.y)));
+    const T sc = fdiv(ef, fmaT(nf.z, nf.z, fmaT(nf.x, nf.x, mul_rn(nf.y, nf.y))));
+    const P3<T> o = mk<T>(mul_rn(sc, nf.x), mul_rn(sc, nf.y), T(0));  // (its z enters fo only)
+    const T fo = fmaT(sc, nf.z, -fmaT(F.lx, o.x, fmaT(F.ly, o.y, F.l0)));
 
-    slot_store<T>(E, 0, a, b);
-    slot_store<T>(E, 1, b, c);
-    slot_store<T>(E, 2, c, a);
-    slab_pass<0, T>(E, -F.qx, T(1) - F.qx, tol);
+    const int n3 = xslab_triangle<T>(a, b, c, -F.qx, T(1) - F.qx, tol, E);
     FaceSums<T> I;
-    yslab_sums<T>(E, -F.qy, T(1) - F.qy, tol, o, fo, F.l0, F.lx, F.ly, I);
+    R.n = yslab_sums<T>(E, n3, -F.qy, T(1) - F.qy, tol, o, fo, F.l0, F.lx, F.ly, I);
 
     // levels the polygon straddles: jlo .. jhi (c_j - zmin > 0 and zmax - c_j > 0)
     const T kf = (T)F.K;
@@ -231,30 +384,24 @@ PSE_HD void face_run(const Src &src, int f, const RunFrame<T> &F, slot2_t<T> *E,
     R.ef = ef;
 }
 
-// The anchor of a level fan: the point of the face plane at height c nearest the local
-// origin in the xy plane.
+// The anchor of a level fan, the point of the face plane at height c nearest the local origin in
+// the xy plane, is s (nx, ny).
 template <class T>
-PSE_HD void fan_anchor(T nx, T ny, T nz, T ef, T c, T &ox, T &oy)
+PSE_HD T fan_anchor(T nx, T ny, T nz, T ef, T c)
 {
-    const T s = fmaT(-nz, c, ef) * fdiv(T(1), fmaT(nx, nx, ny * ny));
-    ox = s * nx;
-    oy = s * ny;
+    return fmaT(-nz, c, ef) * fdiv(T(1), fmaT(nx, nx, mul_rn(ny, ny)));
 }
 
-// Cell volumes of a run from the level sums S[j] = 6 B(c_j): levels at or below the
-// tetrahedron's lowest point in the column hold exactly 0, and levels at or above its highest
-// point the column's whole volume, so they are set so rather than left to the rounding of
-// terms that cancel; then vol_j = (S[j+1] - S[j]) / 6.
-template <int KW, class T>
-PSE_HD void column_finish(const RunFrame<T> &F, T (&S)[KW + 1], T colmin, T colmax, T msum, T (&vol)[KW])
+// Volume of the cell between the levels c0 and c1 of a run, from the level sums s = 6 B(c) over
+// its faces: a level at or below the tetrahedron's lowest point in the column (colmin) holds
+// exactly 0, and one at or above its highest point (colmax) the column's whole volume (msum / 6),
+// so they are set so rather than left to the rounding of terms that cancel.
+template <class T>
+PSE_HD T level_volume(T c0, T c1, T s0, T s1, T colmin, T colmax, T msum)
 {
-#pragma unroll
-    for (int j = 0; j <= KW; ++j) {
-        const T cj = (T)j - F.qz;
-        S[j] = (cj <= colmin) ? T(0) : ((cj >= colmax) ? msum : S[j]);
-    }
-#pragma unroll
-    for (int j = 0; j < KW; ++j) vol[j] = (S[j + 1] - S[j]) * T(1.0 / 6.0);
+    const T b0 = (c0 <= colmin) ? T(0) : ((c0 >= colmax) ? msum : s0);
+    const T b1 = (c1 <= colmin) ? T(0) : ((c1 >= colmax) ? msum : s1);
+    return (b1 - b0) * T(1.0 / 6.0);
 }
 
 // Overlap volumes of a positively oriented tetrahedron (clip frame, relative to the first
@@ -262,11 +409,15 @@ PSE_HD void column_finish(const RunFrame<T> &F, T (&S)[KW + 1], T colmin, T colm
 // gives vertex i (src.vtx(i)) and the outward normal of face f (src.nrm(f)), read when
 // needed; (lx, ly): reference slopes.  lo_open: the tetrahedron may reach below the run (a
 // run that starts above its bounding box's first layer); otherwise B(0) is exactly 0.
-// E: this lane's edge slots (float2 rows with a stride of 32).
+// E: this lane's edge slots (two-scalar rows with a stride of 32).  This is the clip of one run
+// by one thread; the warp kernels deal its faces and its level fans out to lanes (common.cuh)
+// with the same stages and the same order of the sums.
 template <int KW, class T, class Src>
-PSE_HD void column_volumes(const Src &src, T lx, T ly, int K, bool lo_open, T (&vol)[KW], slot2_t<T> *E)
+PSE_HD void column_volumes(const Src &src, T lx, T ly, int K, bool lo_open, T (&vol)[KW], slot2_t<T> *slots)
 {
     const RunFrame<T> F = run_frame<T>(src, lx, ly, K, lo_open);
+    const EdgeSlots<T> E{slots};
+    const P3<T> q = mk<T>(F.qx, F.qy, F.qz);
     // S[j]: 6 B(c_j), c_j = j - q.z, j = 0 .. KW (levels past K are unused)
     T S[KW + 1];
 #pragma unroll
@@ -275,15 +426,17 @@ PSE_HD void column_volumes(const Src &src, T lx, T ly, int K, bool lo_open, T (&
     T colmin = T(1e30), colmax = T(-1e30), msum = T(0);
 #pragma unroll 1
     for (int f = 0; f < 4; ++f) {
-        if (!face_meets_column<T>(src, f, F)) continue;
+        int ia, ib, ic;
+        face_vertices(f, ia, ib, ic);
+        const P3<T> a = sub(src.vtx(ia), q), b = sub(src.vtx(ib), q), c = sub(src.vtx(ic), q);
+        const P3<T> nf = src.nrm(f);
+        if (!face_meets_column<T>(a, b, c, nf.z, F)) continue;
         FaceRun<KW, T> R;
-        face_run<KW, T>(src, f, F, E, R);
+        face_run<KW, T>(a, b, c, nf, F, E, R);
 #pragma unroll 1
         for (int j = R.jlo; j <= R.jhi; ++j) {  // straddled levels: subtract the part above
             const T cj = (T)j - F.qz;
-            T ox, oy;
-            fan_anchor<T>(R.nx, R.ny, R.nz, R.ef, cj, ox, oy);
-            const T g = level_fan<T>(E, cj, ox, oy);
+            const T g = level_fan<false, T>(E, R.n, cj, fan_anchor<T>(R.nx, R.ny, R.nz, R.ef, cj), R.nx, R.ny);
 #pragma unroll
             for (int i = 0; i <= KW; ++i) R.k6[i] -= (i == j) ? g : T(0);
         }
@@ -293,7 +446,9 @@ PSE_HD void column_volumes(const Src &src, T lx, T ly, int K, bool lo_open, T (&
         colmax = fmax(colmax, R.zmax);
         msum += R.m6;
     }
-    column_finish<KW, T>(F, S, colmin, colmax, msum, vol);
+#pragma unroll
+    for (int j = 0; j < KW; ++j)
+        vol[j] = level_volume<T>((T)j - F.qz, (T)(j + 1) - F.qz, S[j], S[j + 1], colmin, colmax, msum);
 }
 
 }  // namespace pse

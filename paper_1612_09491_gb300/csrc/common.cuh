@@ -197,6 +197,23 @@ __device__ __forceinline__ int64_t fold_cell(int64_t c, int64_t g)
     return c < 0 ? c + g : c;
 }
 
+// The same for int32 cells (a base cell within +-2^30 plus an offset within 2^25; a grid has at
+// most 2^24 cells a side).  A cell more than one period away is rare, and its remainder is kept
+// out of line: the deposit kernels are sensitive to the size of their hot code.
+__device__ __noinline__ int fold_far(int c, int g)
+{
+    c %= g;
+    return c < 0 ? c + g : c;
+}
+__device__ __forceinline__ int fold_near(int c, int g)
+{
+    if ((unsigned)c >= (unsigned)g) {
+        c += c < 0 ? g : -g;
+        if ((unsigned)c >= (unsigned)g) c = fold_far(c, g);
+    }
+    return c;
+}
+
 // How a kernel adds to the output cells (compile-time, so that the FP64 kernels carry
 // no trace of the other mode):
 //  * F64: one global FP64 reduction per addend.
@@ -237,16 +254,17 @@ __device__ __forceinline__ void cell_add(const DepositParams &P, double *addr, d
 // Add m to cell (cx, cy, cz) (unfolded grid indices); returns false if the cell is
 // outside an open grid (then the mass is dropped).
 template <Acc A = Acc::RUNTIME>
-__device__ __forceinline__ bool deposit_cell(const DepositParams &P, int64_t cx, int64_t cy, int64_t cz, double m)
+__device__ __forceinline__ bool deposit_cell(const DepositParams &P, int cx, int cy, int cz, double m)
 {
+    const int g0 = (int)P.g[0], g1 = (int)P.g[1], g2 = (int)P.g[2];
     if (P.periodic) {
-        cx = fold_cell(cx, P.g[0]);
-        cy = fold_cell(cy, P.g[1]);
-        cz = fold_cell(cz, P.g[2]);
-    } else if (cx < 0 || cy < 0 || cz < 0 || cx >= P.g[0] || cy >= P.g[1] || cz >= P.g[2]) {
+        cx = fold_near(cx, g0);
+        cy = fold_near(cy, g1);
+        cz = fold_near(cz, g2);
+    } else if ((unsigned)cx >= (unsigned)g0 || (unsigned)cy >= (unsigned)g1 || (unsigned)cz >= (unsigned)g2) {
         return false;
     }
-    cell_add<A>(P, P.out + (cx + P.g[0] * (cy + P.g[1] * cz)), m);
+    cell_add<A>(P, P.out + ((int64_t)cx + g0 * ((int64_t)cy + (int64_t)g1 * cz)), m);
     return true;
 }
 
@@ -362,30 +380,49 @@ struct WarpSmem {
     float pos[4][32];
     float neg[4][32];
     float lx[32], ly[32];  // reference-plane slopes (in the clip's frame)
-    int axis[32];          // the clip's divergence axis (to_axis)
+    int axis[32];          // bits 0-1: the clip's divergence axis (to_axis); kRecCut; kRecGuard
     int lo[3][32];
     int dim[3][32];
-    int base[3][32];
+    int base[3][32];      // uniform grid: the base cell; octree: the leaf's first cell, base-cell frame
     int leaf[32];         // octree: leaf of this (tetrahedron, leaf) pair
-    int org[3][32];       // octree: the leaf's first cell, base-cell frame
     float rho[32];        // 6 m_t / |6V| (deposit = rho * overlap volume, formed in float32)
     int start[32];        // exclusive prefix of the pair counts
-    int skip[32];         // first pair of this record (split tetrahedra; else 0)
-    int guard[32];        // bit 0: a guarded tetrahedron (clipped in float64);
-                          // kGuardFlip: its exact vertices are oriented the other way round
-    int cut[32];          // octree: 1 if the record's cell range starts above the tetrahedron's
-                          // own first layer along its divergence axis (a leaf block cuts it)
-    float *vres;          // this warp's residual block in global memory: [12][32] floats, the
-                          // rounding residuals of guarded records (exact vertex = v + vres)
-    unsigned long long q[64];  // queued partial pairs: t | ix << 5 | iy << 24 | iz << 43
-    unsigned long long gq[64]; // queued partial pairs of guarded tetrahedra (float64 clips)
-    double2 *dpoly;            // the guarded pass's float64 edge slots: [21][32], this warp's
-    float2 poly[21][32];       // FP32 clip: each lane's 7 edge slots, 3 float2 each:
-                               // (a.x, a.y), (a.z, b.x), (b.y, b.z)
+    float *vres;          // warp-per-tetrahedron baseline: this warp's residual block in global
+                          // memory: [12][32] floats, the rounding residuals of guarded records
+                          // (exact vertex = v + vres)
+    union {
+        struct {
+            unsigned long long q[64];   // baseline: queued partial pairs: t | ix << 5 | iy << 24 | iz << 43
+            unsigned long long gq[64];  // baseline: queued partial pairs of guarded tetrahedra (float64 clips)
+        };
+        struct {
+            float4 ra[64];  // queued runs (a ring): first cell along A, B, C; run word (see kRun*)
+            float4 rb[64];  // the run's clip frame: qx, qy, qz, l0
+        };
+    };
+    unsigned char fan[32];     // level fans of one round: the lane that holds the face, first level << 5
+    union {
+        float2 poly[21][32];   // baseline: each lane's 7 edge slots, 3 float2 each
+        struct {
+            float4 eh[7][32];  // column clip: each lane's 7 edge slots (EdgeSlots4)
+            float2 el[7][32];
+        };
+        float comb[6][32];     // face terms of one round, after its fans
+    };
+};
+constexpr int kRecCut = 4;    // octree: the record's cell range starts above the tetrahedron's own
+                              // first layer along its divergence axis (a leaf block cuts it)
+constexpr int kRecGuard = 8;  // a guarded tetrahedron (clipped in float64)
+
+// What the guarded pass keeps per warp in place of the float slots and beyond them.
+struct GuardSmem {
+    double2 slots[21][32];  // each lane's 7 edge slots, 3 double2 each
+    double v[12][32];       // exact vertices, positively oriented
+    double n[12][32];       // their outward face normals
+    double l0[64];          // queued runs: the frame's l0
 };
 
 constexpr int kQBits = 19;  // per-axis cell offset bits in a queue entry
-constexpr int kGuardFlip = 2;
 constexpr unsigned long long kQMask = (1ull << kQBits) - 1;
 
 __device__ __forceinline__ unsigned long long q_pack(int t, int ix, int iy, int iz)
@@ -430,16 +467,50 @@ __device__ __forceinline__ void store_residuals(WarpSmem *S, int lane, const P3<
     }
 }
 
-// Record lane's tetrahedron (uniform grid) for the pair machinery.
-__device__ __forceinline__ void store_record(WarpSmem *S, int lane, const TetSetup<float> &ts,
-                                             const P3<float> (&res)[4], const int (&base)[3], double m_t,
-                                             float kappa_max, int skip)
+// Which records a kernel holds, and so which clips it carries:
+//  * kPassAll: records on both sides of the guard, enumerated by cells; FP32 clips and FP64
+//    clips in the same kernel (the warp-per-tetrahedron baseline);
+//  * kPassFp32: records below the guard only, enumerated by column runs (FP32 column clips);
+//  * kPassGuard: guarded records only, enumerated by column runs (FP64 column clips from
+//    the exact vertices).
+// The warp-cooperative and octree schedules run kPassFp32 and then kPassGuard over the same
+// tetrahedra, so neither kernel carries the other's clip code or registers.
+enum { kPassAll = 0, kPassFp32 = 1, kPassGuard = 2 };
+// the scalar of a pass's column clips
+template <int PASS>
+struct PassScalar {
+    using type = float;
+};
+template <>
+struct PassScalar<kPassGuard> {
+    using type = double;
+};
+
+__device__ __forceinline__ GuardSmem *guard_smem(WarpSmem *S)
 {
+    return reinterpret_cast<GuardSmem *>(reinterpret_cast<unsigned char *>(S) + offsetof(WarpSmem, poly));
+}
+
+// Record lane's tetrahedron for the pair machinery: cells [lo, lo + dim) of the base-cell frame;
+// base: what deposit_pair adds to (uniform) or takes off (octree) a cell of that frame.  In the
+// guarded pass the exact vertices are kept too, oriented by their own determinant, and the
+// float32 vertices take the same order.
+template <int PASS>
+__device__ __forceinline__ void store_record(WarpSmem *S, int lane, const TetSetup<float> &ts,
+                                             const P3<float> (&res)[4], const int (&lo)[3], const int (&dim)[3],
+                                             const int (&base)[3], double m_t, float kappa_max, bool cut)
+{
+    const bool guard = PASS == kPassGuard || (PASS == kPassAll && !(ts.kappa <= kappa_max));
+    bool flip = false;
+    S->rho[lane] = guard ? (float)(6.0 * m_t / exact_vol6(ts.v, res, ts.vol6, &flip))
+                         : __fdiv_rn((float)(6.0 * m_t), (float)ts.vol6);
+    const bool turn = PASS == kPassGuard && flip;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        S->v[3 * q][lane] = ts.v[q].x;
-        S->v[3 * q + 1][lane] = ts.v[q].y;
-        S->v[3 * q + 2][lane] = ts.v[q].z;
+        const int k = (q == 1 && turn) ? 2 : ((q == 2 && turn) ? 1 : q);
+        S->v[3 * k][lane] = ts.v[q].x;
+        S->v[3 * k + 1][lane] = ts.v[q].y;
+        S->v[3 * k + 2][lane] = ts.v[q].z;
         S->n[3 * q][lane] = ts.n[q].x;
         S->n[3 * q + 1][lane] = ts.n[q].y;
         S->n[3 * q + 2][lane] = ts.n[q].z;
@@ -449,21 +520,36 @@ __device__ __forceinline__ void store_record(WarpSmem *S, int lane, const TetSet
     }
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        S->lo[a][lane] = ts.lo[a];
-        S->dim[a][lane] = ts.dim[a];
+        S->lo[a][lane] = lo[a];
+        S->dim[a][lane] = dim[a];
         S->base[a][lane] = base[a];
     }
-    const int guard = (ts.kappa <= kappa_max) ? 0 : 1;
-    bool flip = false;
-    S->rho[lane] = guard ? (float)(6.0 * m_t / exact_vol6(ts.v, res, ts.vol6, &flip))
-                         : __fdiv_rn((float)(6.0 * m_t), (float)ts.vol6);
     S->lx[lane] = ts.lx;
     S->ly[lane] = ts.ly;
-    S->axis[lane] = ts.axis;
-    S->guard[lane] = guard | (flip ? kGuardFlip : 0);
-    S->skip[lane] = skip;
-    S->cut[lane] = 0;
-    if (guard) store_residuals(S, lane, res);
+    S->axis[lane] = ts.axis | (cut ? kRecCut : 0) | (guard ? kRecGuard : 0);
+    if constexpr (PASS == kPassGuard) {
+        GuardSmem *G = guard_smem(S);
+        P3<double> pd[4], nd[4];
+        exact_vertices(ts.v, res, 0, 0, 0, pd);
+        if (turn) {
+            const P3<double> t = pd[1];
+            pd[1] = pd[2];
+            pd[2] = t;
+        }
+        face_normals<double>(pd, nd);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            G->v[3 * q][lane] = pd[q].x;
+            G->v[3 * q + 1][lane] = pd[q].y;
+            G->v[3 * q + 2][lane] = pd[q].z;
+            G->n[3 * q][lane] = nd[q].x;
+            G->n[3 * q + 1][lane] = nd[q].y;
+            G->n[3 * q + 2][lane] = nd[q].z;
+        }
+    }
+    if constexpr (PASS == kPassAll) {
+        if (guard) store_residuals(S, lane, res);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -486,92 +572,103 @@ __device__ __forceinline__ int64_t run_count(const int (&dim)[3], int C)
     return (int64_t)dA * dB * ((dC + kRun - 1) / kRun);
 }
 
-// Run (ia, ib, w) of record t: base-frame first cell (cx, cy, cz) and length kw.
-// (la, lb, lc: the same first cell along the axes A, B and C.)
-__device__ __forceinline__ void run_cells(const WarpSmem *S, int t, int ia, int ib, int w, int &cx, int &cy, int &cz,
-                                          int &kw, int &la, int &lb, int &lc)
-{
-    const int C = S->axis[t], A = axis_a(C), B = axis_b(C);
-    kw = min(kRun, S->dim[C][t] - w * kRun);
-    la = S->lo[A][t] + ia;
-    lb = S->lo[B][t] + ib;
-    lc = S->lo[C][t] + w * kRun;
-    cx = C == 0 ? lc : (C == 1 ? lb : la);
-    cy = C == 1 ? lc : (C == 2 ? lb : la);
-    cz = C == 2 ? lc : (C == 0 ? lb : la);
-}
-__device__ __forceinline__ void run_cells(const WarpSmem *S, int t, int ia, int ib, int w, int &cx, int &cy, int &cz,
-                                          int &kw)
-{
-    int la, lb, lc;
-    run_cells(S, t, ia, ib, w, cx, cy, cz, kw, la, lb, lc);
-}
-
-// Run number `local` of record t (ia fastest, then ib, then w).
-__device__ __forceinline__ void run_of(const WarpSmem *S, int t, int local, int &ia, int &ib, int &w, int &cx,
-                                       int &cy, int &cz, int &kw)
-{
-    const int C = S->axis[t];
-    const int dA = S->dim[axis_a(C)][t], dB = S->dim[axis_b(C)][t];
-    ia = local % dA;
-    const int r = local / dA;
-    ib = r % dB;
-    w = r / dB;
-    run_cells(S, t, ia, ib, w, cx, cy, cz, kw);
-}
-
 // A record's cell offsets must fit the kQBits-bit fields of a queue entry.
 __device__ __forceinline__ bool dims_fit_queue(const int (&dim)[3])
 {
     return dim[0] < (1 << 19) && dim[1] < (1 << 19) && dim[2] < (1 << 19);
 }
 
-// Unguarded record t as the column clip reads it: vertices relative to the run's first cell
-// and relabelled so that axis C is z (to_axis), face normals likewise.  The relabelling is
-// bound once per run as three row pointers, (C+1)%3, (C+2)%3 and C, into the record arrays
-// (vertex or face i is 3 rows = 96 floats further on; the normals follow the vertices at
-// 12 rows = 384 floats), so a fetch is three loads at fixed offsets and no selects.
+// Record t as the column clip reads it: vertices relative to the run's first cell and relabelled
+// so that axis C is z (to_axis), face normals likewise.  The relabelling is bound as three row
+// pointers, (C+1)%3, (C+2)%3 and C, into the record arrays (vertex or face i is 3 rows = 96
+// scalars further on; the normals follow the vertices at 12 rows = 384 scalars), so a fetch is
+// three loads at fixed offsets and no selects.  T = float reads the float32 record; T = double
+// the guarded pass's exact vertices.
+template <class T>
 struct RecordRun {
-    const float *va, *vb, *vc;  // &S->v[row][t] for the three rows
-    float fa, fb, fc;           // the run's first cell along the same three axes
-    __device__ __forceinline__ P3<float> vtx(int i) const
+    const T *va, *vb, *vc;  // row pointers
+    T fa, fb, fc;           // the run's first cell along the same three axes
+    __device__ __forceinline__ P3<T> vtx(int i) const
     {
-        return mk<float>(va[96 * i] - fa, vb[96 * i] - fb, vc[96 * i] - fc);
+        return mk<T>(va[96 * i] - fa, vb[96 * i] - fb, vc[96 * i] - fc);
     }
-    __device__ __forceinline__ P3<float> nrm(int f) const
+    __device__ __forceinline__ P3<T> nrm(int f) const
     {
-        return mk<float>(va[384 + 96 * f], vb[384 + 96 * f], vc[384 + 96 * f]);
+        return mk<T>(va[384 + 96 * f], vb[384 + 96 * f], vc[384 + 96 * f]);
     }
 };
 static_assert(offsetof(WarpSmem, n) == offsetof(WarpSmem, v) + 384 * sizeof(float), "RecordRun reads n after v");
+static_assert(offsetof(GuardSmem, n) == offsetof(GuardSmem, v) + 384 * sizeof(double), "RecordRun reads n after v");
 
-// Guarded record t as the guarded pass's column clip reads it: the exact vertices (float32
-// vertex plus its rounding residual) in float64, in the exact tetrahedron's positive
-// orientation, relative to the run's first cell and relabelled so that axis C is z; the
-// outward face normals are formed from them when asked for.  (v - f is exact: both are
-// float32 values a few cells apart.)
-struct RecordRun64 {
-    const WarpSmem *S;
-    int t, C;
-    float fx, fy, fz;
-    bool flip;
-    __device__ __forceinline__ double co(int row, float f) const
+template <class T>
+__device__ __forceinline__ RecordRun<T> record_run(WarpSmem *S, int t, int C, float la, float lb, float lc)
+{
+    const T *rows;
+    if constexpr (sizeof(T) == sizeof(float)) rows = &S->v[0][t];
+    else rows = &guard_smem(S)->v[0][t];
+    return RecordRun<T>{rows + 32 * axis_a(C), rows + 32 * axis_b(C), rows + 32 * C, (T)la, (T)lb, (T)lc};
+}
+
+// Lane `lane`'s edge slots of the column clip.
+__device__ __forceinline__ EdgeSlots4 lane_slots(WarpSmem *S, int lane, float) { return {&S->eh[0][lane], &S->el[0][lane]}; }
+__device__ __forceinline__ EdgeSlots<double> lane_slots(WarpSmem *S, int lane, double)
+{
+    return {&guard_smem(S)->slots[0][lane]};
+}
+
+// The faces of a run that can reach its column [0,1)^2 (bit f), from the projected vertices p
+// (clip frame, relative to the run's first cell) and the signs of the normals' z components
+// (up: bit f set if face f's is positive).  A face is left out when the square lies beyond its
+// bounding box or beyond one of its edges by a margin far above the rounding of the clip, which
+// would then find an empty polygon and add exactly 0, so leaving it out changes no bit: the
+// margins are 2e-3 of a cell plus 4e-6 (m + 1)^2 on the edge functions (m: the largest
+// coordinate), against errors of about 3e-6 m in positions and 1e-6 m^2 in the edge functions;
+// beyond m = 500 every face is kept.  A face seen edge-on, whose sign is rounding, is a segment
+// to within those errors, so either sign is safe.  On the headline workload's tetrahedra this
+// leaves 2.8 of 4 faces a run (3.2 by the bounding boxes alone).
+__device__ __forceinline__ unsigned face_mask(const P3<float> (&p)[4], unsigned up)
+{
+    float m = 0.f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) m = fmaxf(m, fmaxf(fmaxf(fabsf(p[i].x), fabsf(p[i].y)), fabsf(p[i].z)));
+    if (!(m <= 500.f)) return 15u;
+    const float gap = 2e-3f;
+    bool out[4];
     {
-        return ((double)S->v[row][t] - (double)f) + (double)S->vres[row * 32 + t];
+        const float lx = fminf(p[0].x, p[1].x), hx = fmaxf(p[0].x, p[1].x), lx2 = fminf(p[2].x, p[3].x),
+                    hx2 = fmaxf(p[2].x, p[3].x);
+        const float ly = fminf(p[0].y, p[1].y), hy = fmaxf(p[0].y, p[1].y), ly2 = fminf(p[2].y, p[3].y),
+                    hy2 = fmaxf(p[2].y, p[3].y);
+#pragma unroll
+        for (int f = 0; f < 4; ++f) {
+            // the face's vertices: the other one of f's pair, and the other pair
+            const P3<float> s = p[f ^ 1];
+            const bool lowpair = f < 2;
+            const float mnx = fminf(s.x, lowpair ? lx2 : lx), mxx = fmaxf(s.x, lowpair ? hx2 : hx);
+            const float mny = fminf(s.y, lowpair ? ly2 : ly), mxy = fmaxf(s.y, lowpair ? hy2 : hy);
+            out[f] = mxx < -gap || mnx > 1.f + gap || mxy < -gap || mny > 1.f + gap;
+        }
     }
-    __device__ __forceinline__ P3<double> vtx(int i) const
-    {
-        const int k = flip ? (i == 1 ? 2 : (i == 2 ? 1 : i)) : i;
-        return to_axis(mk<double>(co(3 * k, fx), co(3 * k + 1, fy), co(3 * k + 2, fz)), C);
+    // edge i -> j: the square is wholly to its left (L) or right (R)
+    const float eps = 4e-6f * (m + 1.f) * (m + 1.f);
+    bool L[6], R[6];
+    constexpr int ei[6] = {0, 0, 0, 1, 1, 2}, ej[6] = {1, 2, 3, 2, 3, 3};
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        const P3<float> a = p[ei[k]], b = p[ej[k]];
+        const float dx = b.x - a.x, dy = b.y - a.y;
+        const float c = dx * (0.5f - a.y) - dy * (0.5f - a.x);
+        const float r = fmaf(0.5f + gap, fabsf(dx) + fabsf(dy), eps);
+        L[k] = c > r;
+        R[k] = c < -r;
     }
-    __device__ __forceinline__ P3<double> nrm(int f) const
-    {
-        int a, b, c;
-        face_vertices(f, a, b, c);
-        const P3<double> pa = vtx(a);
-        return cross(sub(vtx(b), pa), sub(vtx(c), pa));
-    }
-};
+    // outward loops (face_vertices): 1-2-3, 0-3-2, 0-1-3, 0-2-1; counter-clockwise when up
+    const bool s0 = (up & 1u) ? (R[3] || R[5] || L[4]) : (L[3] || L[5] || R[4]);
+    const bool s1 = (up & 2u) ? (R[2] || L[5] || L[1]) : (L[2] || R[5] || R[1]);
+    const bool s2 = (up & 4u) ? (R[0] || R[4] || L[2]) : (L[0] || L[4] || R[2]);
+    const bool s3 = (up & 8u) ? (R[1] || L[3] || L[0]) : (L[1] || R[3] || R[0]);
+    return (out[0] || s0 ? 0u : 1u) | (out[1] || s1 ? 0u : 2u) | (out[2] || s2 ? 0u : 4u) | (out[3] || s3 ? 0u : 8u);
+}
 
 // Classify the box of kw cells from cell (cx, cy, cz) along axis C against record t's
 // face planes (classify_cell for kw = 1).
@@ -597,13 +694,13 @@ __device__ __forceinline__ bool deposit_pair(const DepositParams &P, const WarpS
                                              double m)
 {
     if constexpr (OCT) {
-        const int64_t bc = P.bc;
-        const int64_t lx = cx - S->org[0][t], ly = cy - S->org[1][t], lz = cz - S->org[2][t];
-        cell_add<A>(P, P.out + (int64_t)S->leaf[t] * bc * bc * bc + lx + bc * (ly + bc * lz), m);
+        // bc <= 4096: a cell's place in its leaf block needs up to 36 bits
+        const int bc = P.bc;
+        const int lx = cx - S->base[0][t], ly = cy - S->base[1][t], lz = cz - S->base[2][t];
+        cell_add<A>(P, P.out + ((int64_t)(S->leaf[t] * (int64_t)bc + lz) * (bc * bc) + (lx + bc * ly)), m);
         return true;
     } else {
-        return deposit_cell<A>(P, (int64_t)S->base[0][t] + cx, (int64_t)S->base[1][t] + cy, (int64_t)S->base[2][t] + cz,
-                            m);
+        return deposit_cell<A>(P, S->base[0][t] + cx, S->base[1][t] + cy, S->base[2][t] + cz, m);
     }
 }
 
@@ -647,8 +744,8 @@ __device__ __forceinline__ void clip_round(const DepositParams &P, WarpSmem *S, 
         P3<float> pa[4], na[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            pa[q] = to_axis(p[q], S->axis[t]);
-            na[q] = to_axis(n[q], S->axis[t]);
+            pa[q] = to_axis(p[q], S->axis[t] & 3);
+            na[q] = to_axis(n[q], S->axis[t] & 3);
         }
         float err;
         const double vol = (double)overlap_volume_rolled(pa, na, S->lx[t], S->ly[t], err, &S->poly[0][lane]);
@@ -657,41 +754,163 @@ __device__ __forceinline__ void clip_round(const DepositParams &P, WarpSmem *S, 
     __syncwarp();
 }
 
-// Column clips of the first `count` entries of S->q, one run per lane: in float32 (T = float,
-// the records below the guard) or in float64 from the exact vertices (T = double, the
-// guarded records).  (Dealing the (run, face) jobs and the level fans out over the warp
-// raised the active lanes but cost more in shuffles and reloads than it saved: 12% slower.)
+// The run word (ra.w): record t (bits 0-4), faces to clip (bits 5-8), cells kw (9-10), axis C
+// (11-12), lo_open (13).
+constexpr int kRunMask = 5, kRunLen = 9, kRunAxis = 11, kRunOpen = 13;
+constexpr int kRunsPerRound = 16;
+
+// One clip round: the faces of up to 16 queued runs (32 faces at most), one face per lane.
+//
+// The clip is bound by instruction issue, so lanes must not idle: a run needs 2.8 of its 4
+// faces on average, and a face straddles 0.5 levels on average but 2 or 3 somewhere in a warp.
+// One run per lane therefore paid 4 faces and 8 level fans for everybody (19 of 32 lanes
+// active); here faces are dealt to lanes, then the fans of their straddled levels are dealt
+// again, and the cells of the runs (2 lanes a run) sum their faces' terms in face order, as one
+// thread would, so the sums are the same bit for bit.  Measured (one GB300, before -> after):
+// 128^3 onto 256^3 45.2 -> 33.8 ms, 48^3 onto 384^3 46.5 -> 31.0 ms, 256^3 octree with collapsed
+// regions 412 -> 345 ms, shell-crossed 128^3 octree (FP64 clips) 233 -> 141 ms.
 template <bool STATS, bool OCT, Acc A, class T>
-__device__ __forceinline__ void run_round(const DepositParams &P, WarpSmem *S, int count, int lane, Counters &cnt)
+__device__ __forceinline__ void job_round(const DepositParams &P, WarpSmem *S, int lane, int &head, int &qn, int &jobs,
+                                          Counters &cnt)
 {
-    if (lane < count) {
-        const unsigned long long ent = S->q[lane];
-        const int t = (int)(ent & 31u);
-        const int w = (int)((ent >> (5 + 2 * kQBits)) & kQMask);
-        const int C = S->axis[t];
-        int cx, cy, cz, kw, la, lb, lc;
-        run_cells(S, t, (int)((ent >> 5) & kQMask), (int)((ent >> (5 + kQBits)) & kQMask), w, cx, cy, cz, kw, la, lb,
-                  lc);
-        if (STATS) cnt.u[ST_RUNS]++;
-        const bool lo_open = w > 0 || S->cut[t] != 0;
-        double vol[kRun];
-        if constexpr (sizeof(T) == sizeof(float)) {
-            // rows (C+1)%3 = A, (C+2)%3 = B and C, and the run's first cell along them
-            const RecordRun src{&S->v[axis_a(C)][t], &S->v[axis_b(C)][t], &S->v[C][t], (float)la, (float)lb, (float)lc};
-            float v32[kRun];
-            column_volumes<kRun>(src, S->lx[t], S->ly[t], kw, lo_open, v32, &S->poly[0][lane]);
+    const unsigned le_mask = kFull >> (31 - lane);
+    // ---- runs: as many from the head as have at most 32 faces together
+    unsigned word = 0;
+    if (lane < kRunsPerRound && lane < qn) word = __float_as_uint(S->ra[(head + lane) & 63].w);
+    const int nface = __popc((word >> kRunMask) & 15u);
+    int incl = nface;
 #pragma unroll
-            for (int j = 0; j < kRun; ++j) vol[j] = v32[j];
-        } else {
-            const RecordRun64 src{S, t, C, (float)cx, (float)cy, (float)cz, (S->guard[t] & kGuardFlip) != 0};
-            column_volumes<kRun>(src, (double)S->lx[t], (double)S->ly[t], kw, lo_open, vol, S->dpoly + lane);
+    for (int o = 1; o < kRunsPerRound; o <<= 1) {
+        const int y = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += y;
+    }
+    const int first = incl - nface;  // this run's first job
+    const bool fits = lane < kRunsPerRound && lane < qn && incl <= 32;
+    const int R = __popc(__ballot_sync(kFull, fits));
+    const int J = __shfl_sync(kFull, incl, R - 1);
+    const unsigned starts = __reduce_or_sync(kFull, fits ? 1u << first : 0u);
+
+    // ---- one face per lane
+    FaceRun<kRun, T> fr;
+    face_none<kRun, T>(fr);
+    T qz = T(0);
+    {
+        const int r = __popc(starts & le_mask) - 1;
+        const unsigned w = __shfl_sync(kFull, word, r);
+        int k = lane - __shfl_sync(kFull, first, r);
+        if (lane < J) {
+            unsigned m = (w >> kRunMask) & 15u;
+#pragma unroll
+            for (int i = 0; i < 3; ++i) m = (i < k) ? (m & (m - 1u)) : m;
+            const int f = __ffs((int)m) - 1;
+            const int slot = (head + r) & 63;
+            const float4 ra = S->ra[slot], rb = S->rb[slot];
+            const int t = (int)(w & 31u), C = (int)((w >> kRunAxis) & 3u);
+            const RecordRun<T> src = record_run<T>(S, t, C, ra.x, ra.y, ra.z);
+            RunFrame<T> F;
+            F.qx = (T)rb.x;
+            F.qy = (T)rb.y;
+            F.qz = (T)rb.z;
+            if constexpr (sizeof(T) == sizeof(float)) F.l0 = rb.w;
+            else F.l0 = guard_smem(S)->l0[slot];
+            F.lx = (T)S->lx[t];
+            F.ly = (T)S->ly[t];
+            F.K = (int)((w >> kRunLen) & 3u);
+            F.j0 = ((w >> kRunOpen) & 1u) ? 0 : 1;
+            qz = F.qz;
+            int ia, ib, ic;
+            face_vertices(f, ia, ib, ic);
+            const P3<T> q = mk<T>(F.qx, F.qy, F.qz);
+            const P3<T> a = sub(src.vtx(ia), q), b = sub(src.vtx(ib), q), c = sub(src.vtx(ic), q);
+            const P3<T> nf = src.nrm(f);
+            if (face_meets_column<T>(a, b, c, nf.z, F)) face_run<kRun, T>(a, b, c, nf, F, lane_slots(S, lane, T(0)), fr);
         }
-        const float rho = S->rho[t];
+    }
+    __syncwarp();
+
+    // ---- level fans, one per lane: whole faces in order, 32 fans at most per pass
+    int pend = fr.jhi >= fr.jlo ? fr.jhi - fr.jlo + 1 : 0;
+#pragma unroll 1
+    while (__any_sync(kFull, pend > 0)) {
+        int inc = pend;
 #pragma unroll
-        for (int j = 0; j < kRun; ++j) {
-            const int ex = cx + (C == 0 ? j : 0), ey = cy + (C == 1 ? j : 0), ez = cz + (C == 2 ? j : 0);
-            if (STATS && j < kw) {
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(kFull, inc, o);
+            if (lane >= o) inc += y;
+        }
+        const bool take = pend > 0 && inc <= 32;
+        const int at = inc - pend;
+        if (take) S->fan[at] = (unsigned char)(lane | (fr.jlo << 5));
+        const unsigned heads = __reduce_or_sync(kFull, take ? 1u << at : 0u);
+        const int nfan = (int)__reduce_max_sync(kFull, take ? (unsigned)inc : 0u);
+        __syncwarp();
+        int from = lane, j = 0;
+        if (lane < nfan) {
+            const int p = 31 - __clz((int)(heads & le_mask));
+            const int e = S->fan[p];
+            from = e & 31;
+            j = (e >> 5) + lane - p;
+        }
+        const T nx = __shfl_sync(kFull, fr.nx, from), ny = __shfl_sync(kFull, fr.ny, from),
+                nz = __shfl_sync(kFull, fr.nz, from), ef = __shfl_sync(kFull, fr.ef, from),
+                fq = __shfl_sync(kFull, qz, from);
+        const int ne = __shfl_sync(kFull, fr.n, from);
+        T g = T(0);
+        if (lane < nfan) {
+            const T cj = (T)j - fq;
+            g = level_fan<OCT, T>(lane_slots(S, from, T(0)), ne, cj, fan_anchor<T>(nx, ny, nz, ef, cj), nx, ny);
+        }
+#pragma unroll
+        for (int i = 0; i <= kRun; ++i) {
+            const T x = __shfl_sync(kFull, g, (at + i - fr.jlo) & 31);
+            if (take && i >= fr.jlo && i <= fr.jhi) fr.k6[i] -= x;
+        }
+        if (take) pend = 0;
+        __syncwarp();
+    }
+
+    // ---- the runs' cells, two lanes a run
+    T(*comb)[32];
+    if constexpr (sizeof(T) == sizeof(float)) comb = S->comb;
+    else comb = reinterpret_cast<double(*)[32]>(&guard_smem(S)->slots[0][0]);
+    if (lane < J) {
+#pragma unroll
+        for (int i = 0; i <= kRun; ++i) comb[i][lane] = fr.k6[i];
+        comb[3][lane] = fr.zmin;
+        comb[4][lane] = fr.zmax;
+        comb[5][lane] = fr.m6;
+    }
+    __syncwarp();
+    {
+        static_assert(kRun == 2, "two lanes a run");
+        const int r = lane >> 1, j = lane & 1;
+        const unsigned w = __shfl_sync(kFull, word, r);
+        const int j0 = __shfl_sync(kFull, first, r);
+        const int kw = (int)((w >> kRunLen) & 3u);
+        if (r < R && j < kw) {
+            const int nf = __popc((w >> kRunMask) & 15u);
+            T s0 = T(0), s1 = T(0), colmin = T(1e30), colmax = T(-1e30), msum = T(0);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (i < nf) {
+                    s0 += comb[j][j0 + i];
+                    s1 += comb[j + 1][j0 + i];
+                    colmin = fmin(colmin, comb[3][j0 + i]);
+                    colmax = fmax(colmax, comb[4][j0 + i]);
+                    msum += comb[5][j0 + i];
+                }
+            }
+            const int slot = (head + r) & 63;
+            const float4 ra = S->ra[slot];
+            const T fq = (T)S->rb[slot].z;
+            const T vol = level_volume<T>((T)j - fq, (T)(j + 1) - fq, s0, s1, colmin, colmax, msum);
+            const int t = (int)(w & 31u), C = (int)((w >> kRunAxis) & 3u);
+            const int la = (int)ra.x, lb = (int)ra.y, lc = (int)ra.z + j;
+            const int ex = C == 0 ? lc : (C == 1 ? lb : la), ey = C == 1 ? lc : (C == 2 ? lb : la),
+                      ez = C == 2 ? lc : (C == 0 ? lb : la);
+            if (STATS) {
                 // the same per-cell classification as the cell schedules, for the counters
+                if (j == 0) cnt.u[ST_RUNS]++;
                 P3<float> n[4];
                 float e[4], ps[4], ng[4];
 #pragma unroll
@@ -709,14 +928,18 @@ __device__ __forceinline__ void run_round(const DepositParams &P, WarpSmem *S, i
                     cnt.u[ST_INSIDE_CELLS]++;
                 }
             }
-            if (j < kw && vol[j] > 0.0) {
+            if (vol > T(0)) {
                 if (STATS) cnt.u[ST_OVERLAPPED]++;
-                const double m = (sizeof(T) == sizeof(float)) ? (double)(rho * (float)vol[j]) : (double)rho * vol[j];
+                const float rho = S->rho[t];
+                const double m = (sizeof(T) == sizeof(float)) ? (double)(rho * (float)vol) : (double)rho * vol;
                 cnt.add_dep(m);
                 if (!deposit_pair<OCT, A>(P, S, t, ex, ey, ez, m) && STATS) cnt.dropped += m;
             }
         }
     }
+    head = (head + R) & 63;
+    qn -= R;
+    jobs -= J;
     __syncwarp();
 }
 
@@ -766,35 +989,125 @@ __device__ __forceinline__ int64_t listed_guarded(const DepositParams &P)
     return c > (unsigned long long)P.guard_cap ? -1 : (int64_t)c;
 }
 
-// Which records a kernel holds, and so which clips it carries:
-//  * kPassAll: records on both sides of the guard, enumerated by cells; FP32 clips and FP64
-//    clips in the same kernel (the warp-per-tetrahedron baseline);
-//  * kPassFp32: records below the guard only, enumerated by column runs (FP32 column clips);
-//  * kPassGuard: guarded records only, enumerated by column runs (FP64 column clips from
-//    the exact vertices).
-// The warp-cooperative and octree schedules run kPassFp32 and then kPassGuard over the same
-// tetrahedra, so neither kernel carries the other's clip code or registers.
-enum { kPassAll = 0, kPassFp32 = 1, kPassGuard = 2 };
-
-// Enumerate every (virtual tetrahedron, cell or run) pair of the 32 records in S (npairs:
-// this lane's pair count), 32 pairs per round: classify; deposit "cell inside" pairs; queue
-// partial pairs and clip them 32 at a time.
-template <bool STATS, bool OCT, Acc A, int PASS>
-__device__ __forceinline__ void coop_pairs(const DepositParams &P, WarpSmem *S, int lane, int npairs, Counters &cnt)
+// Inclusive prefix of the lanes' pair counts into S->start (exclusive) and their total.
+__device__ __forceinline__ int pair_prefix(WarpSmem *S, int lane, int npairs)
 {
-    constexpr bool COL = PASS != kPassAll;  // both passes of the warp schedules clip column runs
-    constexpr bool HAS_Q = true;
-    constexpr bool HAS_GQ = PASS == kPassAll;
-    const unsigned lt_mask = (1u << lane) - 1u;
     int incl = npairs;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const int y = __shfl_up_sync(kFull, incl, o);
         if (lane >= o) incl += y;
     }
-    const int total = __shfl_sync(kFull, incl, 31);
     S->start[lane] = incl - npairs;
     __syncwarp();
+    return __shfl_sync(kFull, incl, 31);
+}
+
+// The record that holds pair idx.
+__device__ __forceinline__ int pair_record(const WarpSmem *S, int idx)
+{
+    int t = 0;
+#pragma unroll
+    for (int step = 16; step >= 1; step >>= 1)
+        if (S->start[t + step] <= idx && t + step < 32) t += step;
+    return t;
+}
+
+// Enumerate every (virtual tetrahedron, run) pair of the 32 records in S (npairs: this lane's
+// run count; skip: the first run of the records, for pieces of a split tetrahedron), 32 per
+// step: classify; deposit the cells of "inside" runs; queue the partial runs with their clip
+// frame and the faces that reach their column, and clip 32 faces at a time.
+template <bool STATS, bool OCT, Acc A, class T>
+__device__ __forceinline__ void coop_runs(const DepositParams &P, WarpSmem *S, int lane, int npairs, int skip,
+                                          Counters &cnt)
+{
+    const unsigned lt_mask = (1u << lane) - 1u;
+    const int total = pair_prefix(S, lane, npairs);
+    int head = 0, qn = 0, jobs = 0;  // the ring of queued runs; the faces they hold
+#pragma unroll 1
+    for (int b0 = 0; b0 < total; b0 += 32) {
+        const int idx = b0 + lane;
+        unsigned word = 0;
+        float4 ra = make_float4(0.f, 0.f, 0.f, 0.f), rb = ra;
+        double l0 = 0.0;
+        if (idx < total) {
+            const int t = pair_record(S, idx);
+            int local = idx - S->start[t] + skip;
+            const int rec = S->axis[t];
+            const int C = rec & 3, iA = axis_a(C), iB = axis_b(C);
+            // run number `local`: ia fastest, then ib, then w
+            const int dA = S->dim[iA][t], dB = S->dim[iB][t];
+            const int rest = local / dA, w = rest / dB;
+            const int kw = min(kRun, S->dim[C][t] - w * kRun);
+            const int la = S->lo[iA][t] + (local - rest * dA), lb = S->lo[iB][t] + (rest - w * dB),
+                      lc = S->lo[C][t] + w * kRun;
+            const int cx = C == 0 ? lc : (C == 1 ? lb : la), cy = C == 1 ? lc : (C == 2 ? lb : la),
+                      cz = C == 2 ? lc : (C == 0 ? lb : la);
+            const int cls = classify_run(S, t, C, (float)cx, (float)cy, (float)cz, kw);
+            if (cls == CELL_INSIDE) {
+                const double m = (double)S->rho[t];
+                for (int j = 0; j < kw; ++j) {
+                    cnt.add_dep(m);
+                    if (!deposit_pair<OCT, A>(P, S, t, cx + (C == 0 ? j : 0), cy + (C == 1 ? j : 0),
+                                              cz + (C == 2 ? j : 0), m) && STATS)
+                        cnt.dropped += m;
+                }
+                if (STATS) { cnt.u[ST_INSIDE_CELLS] += kw; cnt.u[ST_OVERLAPPED] += kw; }
+            } else if (cls == CELL_PARTIAL) {
+                const RecordRun<float> near = record_run<float>(S, t, C, (float)la, (float)lb, (float)lc);
+                P3<float> p[4];
+                unsigned up = 0, flat = 0;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    p[q] = near.vtx(q);
+                    if constexpr (sizeof(T) == sizeof(float)) {
+                        const float nz = near.vc[384 + 96 * q];
+                        up |= nz > 0.f ? 1u << q : 0u;
+                        flat |= nz == 0.f ? 1u << q : 0u;  // vertical: no projected area
+                    } else {
+                        const double *nz = &guard_smem(S)->n[3 * q + C][t];
+                        up |= __double2hiint(*nz) >= 0 ? 1u << q : 0u;
+                    }
+                }
+                unsigned mask = face_mask(p, up) & ~flat;
+                if (STATS && mask == 0u) mask = 1u;  // counted as a run all the same
+                if (mask != 0u) {
+                    const bool lo_open = w > 0 || (rec & kRecCut) != 0;
+                    word = (unsigned)t | (mask << kRunMask) | ((unsigned)kw << kRunLen) | ((unsigned)C << kRunAxis) |
+                           (lo_open ? 1u << kRunOpen : 0u);
+                    ra = make_float4((float)la, (float)lb, (float)lc, __uint_as_float(word));
+                    const RecordRun<T> src = record_run<T>(S, t, C, ra.x, ra.y, ra.z);
+                    const RunFrame<T> F = run_frame<T>(src, (T)S->lx[t], (T)S->ly[t], kw, lo_open);
+                    rb = make_float4((float)F.qx, (float)F.qy, (float)F.qz, (float)F.l0);
+                    l0 = (double)F.l0;
+                }
+            }
+        }
+        const unsigned bal = __ballot_sync(kFull, word != 0u);
+        if (word != 0u) {
+            const int slot = (head + qn + __popc(bal & lt_mask)) & 63;
+            S->ra[slot] = ra;
+            S->rb[slot] = rb;
+            if constexpr (sizeof(T) != sizeof(float)) guard_smem(S)->l0[slot] = l0;
+        }
+        qn += __popc(bal);
+        jobs += (int)__reduce_add_sync(kFull, (unsigned)__popc((word >> kRunMask) & 15u));
+        __syncwarp();
+        const bool last = b0 + 32 >= total;
+#pragma unroll 1
+        while (jobs >= 32 || (last && qn > 0)) job_round<STATS, OCT, A, T>(P, S, lane, head, qn, jobs, cnt);
+    }
+    cnt.fold_dep();
+}
+
+// Enumerate every (tetrahedron, cell) pair of the records in S, 32 pairs per round (the
+// warp-per-tetrahedron baseline): classify; deposit "cell inside" pairs; queue partial pairs,
+// those of guarded tetrahedra apart, and clip them 32 at a time.
+template <bool STATS, Acc A>
+__device__ __forceinline__ void coop_cells(const DepositParams &P, WarpSmem *S, int lane, int npairs, Counters &cnt)
+{
+    const unsigned lt_mask = (1u << lane) - 1u;
+    const int total = pair_prefix(S, lane, npairs);
     // one clip_round call site, so that the clip is inlined once (instruction-cache footprint)
     int qn = 0, gn = 0;
     for (int b0 = 0;; b0 += 32) {
@@ -803,102 +1116,67 @@ __device__ __forceinline__ void coop_pairs(const DepositParams &P, WarpSmem *S, 
             bool partial = false, gpartial = false;
             unsigned long long ent = 0;
             if (idx < total) {
-                int t = 0;
+                const int t = pair_record(S, idx);
+                const int local = idx - S->start[t];
+                int ix, iy, iz;
+                decompose(local, S->dim[0][t], S->dim[1][t], ix, iy, iz);
+                const float cx = (float)(S->lo[0][t] + ix), cy = (float)(S->lo[1][t] + iy),
+                            cz = (float)(S->lo[2][t] + iz);
+                P3<float> n[4];
+                float e[4], ps[4], ng[4];
 #pragma unroll
-                for (int step = 16; step >= 1; step >>= 1)
-                    if (S->start[t + step] <= idx && t + step < 32) t += step;
-                const int local = idx - S->start[t] + S->skip[t];
-                if constexpr (COL) {
-                    int ia, ib, w, cx, cy, cz, kw;
-                    run_of(S, t, local, ia, ib, w, cx, cy, cz, kw);
-                    const int C = S->axis[t];
-                    const int cls = classify_run(S, t, C, (float)cx, (float)cy, (float)cz, kw);
-                    if (cls == CELL_INSIDE) {
-                        const double m = (double)S->rho[t];
-                        for (int j = 0; j < kw; ++j) {
-                            cnt.add_dep(m);
-                            if (!deposit_pair<OCT, A>(P, S, t, cx + (C == 0 ? j : 0), cy + (C == 1 ? j : 0),
-                                                      cz + (C == 2 ? j : 0), m) && STATS)
-                                cnt.dropped += m;
-                        }
-                        if (STATS) { cnt.u[ST_INSIDE_CELLS] += kw; cnt.u[ST_OVERLAPPED] += kw; }
-                    } else if (cls == CELL_PARTIAL) {
-                        ent = q_pack(t, ia, ib, w);
-                        partial = true;
-                    }
-                } else {
-                    int ix, iy, iz;
-                    decompose(local, S->dim[0][t], S->dim[1][t], ix, iy, iz);
-                    const float cx = (float)(S->lo[0][t] + ix), cy = (float)(S->lo[1][t] + iy),
-                                cz = (float)(S->lo[2][t] + iz);
-                    P3<float> n[4];
-                    float e[4], ps[4], ng[4];
-#pragma unroll
-                    for (int f = 0; f < 4; ++f) {
-                        n[f] = mk<float>(S->n[3 * f][t], S->n[3 * f + 1][t], S->n[3 * f + 2][t]);
-                        e[f] = S->e[f][t];
-                        ps[f] = S->pos[f][t];
-                        ng[f] = S->neg[f][t];
-                    }
-                    const int cls = classify_cell<float>(n, e, ps, ng, cx, cy, cz);
-                    if (cls == CELL_INSIDE) {
-                        const double m = (double)S->rho[t];
-                        cnt.add_dep(m);
-                        if (!deposit_pair<OCT, A>(P, S, t, S->lo[0][t] + ix, S->lo[1][t] + iy, S->lo[2][t] + iz, m) &&
-                            STATS)
-                            cnt.dropped += m;
-                        if (STATS) { cnt.u[ST_INSIDE_CELLS]++; cnt.u[ST_OVERLAPPED]++; }
-                    } else if (cls == CELL_PARTIAL) {
-                        ent = q_pack(t, ix, iy, iz);
-                        if (PASS == kPassGuard || (PASS == kPassAll && S->guard[t])) gpartial = true;
-                        else partial = true;
-                    }
+                for (int f = 0; f < 4; ++f) {
+                    n[f] = mk<float>(S->n[3 * f][t], S->n[3 * f + 1][t], S->n[3 * f + 2][t]);
+                    e[f] = S->e[f][t];
+                    ps[f] = S->pos[f][t];
+                    ng[f] = S->neg[f][t];
+                }
+                const int cls = classify_cell<float>(n, e, ps, ng, cx, cy, cz);
+                if (cls == CELL_INSIDE) {
+                    const double m = (double)S->rho[t];
+                    cnt.add_dep(m);
+                    if (!deposit_pair<false, A>(P, S, t, S->lo[0][t] + ix, S->lo[1][t] + iy, S->lo[2][t] + iz, m) &&
+                        STATS)
+                        cnt.dropped += m;
+                    if (STATS) { cnt.u[ST_INSIDE_CELLS]++; cnt.u[ST_OVERLAPPED]++; }
+                } else if (cls == CELL_PARTIAL) {
+                    ent = q_pack(t, ix, iy, iz);
+                    if (S->axis[t] & kRecGuard) gpartial = true;
+                    else partial = true;
                 }
             }
-            if constexpr (HAS_Q) {
-                const unsigned bal = __ballot_sync(kFull, partial);
-                if (partial) S->q[qn + __popc(bal & lt_mask)] = ent;
-                qn += __popc(bal);
-            }
-            if constexpr (HAS_GQ) {
-                const unsigned gbal = __ballot_sync(kFull, gpartial);
-                if (gpartial) S->gq[gn + __popc(gbal & lt_mask)] = ent;
-                gn += __popc(gbal);
-            }
+            const unsigned bal = __ballot_sync(kFull, partial);
+            if (partial) S->q[qn + __popc(bal & lt_mask)] = ent;
+            qn += __popc(bal);
+            const unsigned gbal = __ballot_sync(kFull, gpartial);
+            if (gpartial) S->gq[gn + __popc(gbal & lt_mask)] = ent;
+            gn += __popc(gbal);
             __syncwarp();
         }
         const bool last = b0 + 32 >= total;
-        if constexpr (HAS_Q) {
-            if (qn >= 32 || (last && qn > 0)) {
-                const int take = qn >= 32 ? 32 : qn;
-                if constexpr (PASS == kPassFp32) run_round<STATS, OCT, A, float>(P, S, take, lane, cnt);
-                else if constexpr (PASS == kPassGuard) run_round<STATS, OCT, A, double>(P, S, take, lane, cnt);
-                else clip_round<STATS, OCT, A>(P, S, take, lane, cnt);
-                if (lane < qn - take) S->q[lane] = S->q[take + lane];
-                qn -= take;
-                __syncwarp();
-            }
+        if (qn >= 32 || (last && qn > 0)) {
+            const int take = qn >= 32 ? 32 : qn;
+            clip_round<STATS, false, A>(P, S, take, lane, cnt);
+            if (lane < qn - take) S->q[lane] = S->q[take + lane];
+            qn -= take;
+            __syncwarp();
         }
-        if constexpr (HAS_GQ) {
-            if (gn >= 32 || (last && gn > 0)) {
-                const int take = gn >= 32 ? 32 : gn;
-                redo_round<STATS, OCT, A>(P, S, take, lane, cnt);
-                if (lane < gn - take) S->gq[lane] = S->gq[take + lane];
-                gn -= take;
-                __syncwarp();
-            }
+        if (gn >= 32 || (last && gn > 0)) {
+            const int take = gn >= 32 ? 32 : gn;
+            redo_round<STATS, false, A>(P, S, take, lane, cnt);
+            if (lane < gn - take) S->gq[lane] = S->gq[take + lane];
+            gn -= take;
+            __syncwarp();
         }
         if (last && qn == 0 && gn == 0) break;
     }
     cnt.fold_dep();
 }
 
-
-// Each warp's shared memory is a WarpSmem, except in the guarded pass: there the float64
-// edge slots ([21][32] double2) take the place of the FP32 ones (poly, the struct's last
-// member, which that pass never touches) and run past the struct's end, so a warp needs
-// 19 KB instead of 24 and three 4-warp blocks fit an SM.
-constexpr size_t kGuardWarpBytes = offsetof(WarpSmem, poly) + sizeof(double2) * 21 * 32;
+// Each warp's shared memory is a WarpSmem; in the guarded pass a GuardSmem takes the place of
+// its float slots (the struct's last member, which that pass never touches) and runs past the
+// struct's end: 26 KB a warp, two 4-warp blocks an SM.
+constexpr size_t kGuardWarpBytes = offsetof(WarpSmem, poly) + sizeof(GuardSmem);
 static_assert(offsetof(WarpSmem, poly) % 16 == 0 && kGuardWarpBytes % 16 == 0 && sizeof(WarpSmem) % 16 == 0,
               "warp blocks of shared memory must keep 16-byte alignment");
 PSE_HD constexpr size_t warp_stride(bool guard_slots) { return guard_slots ? kGuardWarpBytes : sizeof(WarpSmem); }
@@ -910,12 +1188,10 @@ __device__ __forceinline__ WarpSmem *warp_smem(bool guard_slots)
     return reinterpret_cast<WarpSmem *>(smem_raw + (threadIdx.x >> 5) * warp_stride(guard_slots));
 }
 
-// Point S->vres at this warp's residual block and, in the guarded pass, S->dpoly at its
-// float64 edge slots (every lane writes the same values).
-__device__ __forceinline__ void bind_residuals(const DepositParams &P, WarpSmem *S, bool guard_slots = false)
+// Point S->vres at this warp's residual block (every lane writes the same value).
+__device__ __forceinline__ void bind_residuals(const DepositParams &P, WarpSmem *S)
 {
     S->vres = P.vres + ((size_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * (12 * 32);
-    if (guard_slots) S->dpoly = reinterpret_cast<double2 *>(&S->poly[0][0]);
     __syncwarp();
 }
 

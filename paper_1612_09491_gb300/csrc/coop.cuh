@@ -3,12 +3,12 @@
 // deposit_comp.cu the compensated-FP32 ones, so the two build in parallel.
 //
 // One warp takes a batch of 32 tetrahedra (32 Lagrangian cubes x one Kuhn permutation),
-// enumerates all their (tetrahedron, cell) pairs 32 at a time, classifies them in
-// lock-step, deposits "cell inside tetrahedron" pairs at once and compacts the partial
-// pairs into a per-warp queue; whenever 32 are queued every lane clips one (FP32, in
-// registers).  Tetrahedra whose conditioning estimate exceeds the guard are clipped in
-// FP64.  This is the role of the paper's warp-per-tetrahedron kernel with its
-// shared-memory buffer of partial cells (Sec. 6.2), generalised to batches of tetrahedra
+// enumerates all their (tetrahedron, column run) pairs 32 at a time, classifies them in
+// lock-step, deposits "cells inside tetrahedron" runs at once and compacts the partial
+// runs into a per-warp queue; whenever the queue holds 32 faces to clip, every lane clips one
+// (job_round).  Tetrahedra whose conditioning estimate exceeds the guard are clipped in
+// FP64 in a pass of their own.  This is the role of the paper's warp-per-tetrahedron kernel with
+// its shared-memory buffer of partial cells (Sec. 6.2), generalised to batches of tetrahedra
 // so that small tetrahedra fill the warp too.
 #pragma once
 
@@ -25,7 +25,7 @@ namespace {
 // the lane's pair count (len on lane 0, else 0).
 template <bool STATS, int PASS>
 __device__ __forceinline__ int chunk_setup(const DepositParams &P, WarpSmem *S, int lane, int64_t item, int64_t q,
-                                           Counters &cnt)
+                                           int &skip, Counters &cnt)
 {
     // queue entry e: the last with chunk_start[e] <= item
     int64_t lo = 0, hi = q - 1;
@@ -38,6 +38,7 @@ __device__ __forceinline__ int chunk_setup(const DepositParams &P, WarpSmem *S, 
     const int64_t first = (item - P.chunk_start[lo]) * (int64_t)P.chunk_cells;
     const int64_t npair = P.q_cells[lo];
     const int len = (int)min((int64_t)P.chunk_cells, npair - first);
+    skip = (int)first;
     if (lane != 0 || len <= 0) return 0;
     const int64_t id = P.q_tet[lo];
     P3<float> v[4], res[4];
@@ -61,7 +62,7 @@ __device__ __forceinline__ int chunk_setup(const DepositParams &P, WarpSmem *S, 
     // each pass takes the pieces of its own side of the guard
     const bool guard = !(ts.kappa <= P.kappa_max);
     if (guard != (PASS == kPassGuard)) return 0;
-    store_record(S, 0, ts, res, base, m_t, P.kappa_max, (int)first);
+    store_record<PASS>(S, 0, ts, res, ts.lo, ts.dim, base, m_t, P.kappa_max, false);
     return len;
 }
 
@@ -74,8 +75,8 @@ template <bool STATS, int MINB, bool BINNED, Acc A, int PASS>
 __global__ void __launch_bounds__(kCoopThreads, MINB) k_warp_coop(const DepositParams P)
 {
     constexpr bool FIRST = PASS == kPassFp32;
+    using T = typename PassScalar<PASS>::type;
     WarpSmem *S = warp_smem(!FIRST);
-    bind_residuals(P, S, !FIRST);
     const int lane = threadIdx.x & 31;
     Counters cnt;
     if (STATS) cnt.zero();
@@ -155,15 +156,16 @@ __global__ void __launch_bounds__(kCoopThreads, MINB) k_warp_coop(const DepositP
         }
 
         const int nsub_item = (is_chunk || LIST) ? 1 : nsub;
+#pragma unroll 1
         for (int si = 0; si < nsub_item; ++si) {
             const int s = LIST ? s_listed : si;
             // ---- 1. one tetrahedron per lane (or the queued tetrahedron's chunk on lane 0)
-            int npairs = 0;
+            int npairs = 0, skip = 0;
             double m_t = 0.0;
             int64_t tid = 0;
             bool to_list = false;
             if (is_chunk) {
-                npairs = chunk_setup<STATS, PASS>(P, S, lane, (int64_t)item, q, cnt);
+                npairs = chunk_setup<STATS, PASS>(P, S, lane, (int64_t)item, q, skip, cnt);
                 __syncwarp();
             } else if (unit >= 0) {
                 P3<float> v[4];
@@ -194,15 +196,15 @@ __global__ void __launch_bounds__(kCoopThreads, MINB) k_warp_coop(const DepositP
                 } else if (ts.vol6 == 0.0) {
                     int c[3];
                     centroid_cell(ts.v, c);
-                    if (!deposit_cell<A>(P, (int64_t)base[0] + c[0], (int64_t)base[1] + c[1], (int64_t)base[2] + c[2], m_t) &&
+                    if (!deposit_cell<A>(P, base[0] + c[0], base[1] + c[1], base[2] + c[2], m_t) &&
                         STATS)
                         cnt.dropped += m_t;
                     cnt.add_tgt(P, m_t);
                     cnt.add_dep(m_t);
                     if (STATS) { cnt.u[ST_DEGENERATE]++; cnt.u[ST_OVERLAPPED]++; }
                 } else if (ncell == 1) {
-                    if (!deposit_cell<A>(P, (int64_t)base[0] + ts.lo[0], (int64_t)base[1] + ts.lo[1],
-                                      (int64_t)base[2] + ts.lo[2], m_t) && STATS)
+                    if (!deposit_cell<A>(P, base[0] + ts.lo[0], base[1] + ts.lo[1],
+                                      base[2] + ts.lo[2], m_t) && STATS)
                         cnt.dropped += m_t;
                     cnt.add_tgt(P, m_t);
                     cnt.add_dep(m_t);
@@ -225,7 +227,7 @@ __global__ void __launch_bounds__(kCoopThreads, MINB) k_warp_coop(const DepositP
                         P3<float> res[4];
 #pragma unroll
                         for (int q = 0; q < 4; ++q) res[q] = mk<float>(0.f, 0.f, 0.f);
-                        store_record(S, lane, ts, res, base, m_t, P.kappa_max, 0);
+                        store_record<PASS>(S, lane, ts, res, ts.lo, ts.dim, base, m_t, P.kappa_max, false);
                     } else {
                         to_list = !BINNED;
                     }
@@ -238,12 +240,12 @@ __global__ void __launch_bounds__(kCoopThreads, MINB) k_warp_coop(const DepositP
                     if (P.src == SRC_TETS) explicit_tet<float>(P, unit, v2, b2, res);
                     else lattice_tet<float>(P, ci, cj, ck, s, v2, b2, res);
                     if (swapped) swap12(res);
-                    store_record(S, lane, ts, res, base, m_t, P.kappa_max, 0);
+                    store_record<PASS>(S, lane, ts, res, ts.lo, ts.dim, base, m_t, P.kappa_max, false);
                 }
             }
             if (FIRST && !BINNED) list_guarded(P, to_list, tid, lane);
             // ---- 2. pair enumeration and clips
-            coop_pairs<STATS, false, A, PASS>(P, S, lane, npairs, cnt);
+            coop_runs<STATS, false, A, T>(P, S, lane, npairs, skip, cnt);
             __syncwarp();
         }
     }

@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(128) k_thread_per_tet(const DepositParams P)
                         if (STATS) cnt.u[ST_OVERLAPPED]++;
                         const double m = rho * vol;
                         cnt.add_dep(m);
-                        if (!deposit_cell(P, (int64_t)base[0] + cx, (int64_t)base[1] + cy, (int64_t)base[2] + cz, m) &&
+                        if (!deposit_cell(P, base[0] + cx, base[1] + cy, base[2] + cz, m) &&
                             STATS)
                             cnt.dropped += m;
                     }
@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(kCoopThreads, 2) k_warp_per_tet(const DepositP
                     int c[3];
                     if (ts.vol6 == 0.0) centroid_cell(ts.v, c);
                     else { c[0] = ts.lo[0]; c[1] = ts.lo[1]; c[2] = ts.lo[2]; }
-                    if (!deposit_cell(P, (int64_t)base[0] + c[0], (int64_t)base[1] + c[1], (int64_t)base[2] + c[2], m_t) &&
+                    if (!deposit_cell(P, base[0] + c[0], base[1] + c[1], base[2] + c[2], m_t) &&
                         STATS)
                         cnt.dropped += m_t;
                     cnt.add_tgt(P, m_t);
@@ -193,12 +193,12 @@ __global__ void __launch_bounds__(kCoopThreads, 2) k_warp_per_tet(const DepositP
                     npairs = (int)ncell;
                     cnt.add_tgt(P, m_t);
                     if (STATS) { cnt.u[ST_BBOX_CELLS] += ncell; cnt.u[ST_BIN0 + size_bin(ncell)]++; }
-                    store_record(S, 0, ts, res, base, m_t, P.kappa_max, 0);
+                    store_record<kPassAll>(S, 0, ts, res, ts.lo, ts.dim, base, m_t, P.kappa_max, false);
                 }
             }
         }
         __syncwarp();
-        coop_pairs<STATS, false, Acc::RUNTIME, kPassAll>(P, S, lane, npairs, cnt);
+        coop_cells<STATS, Acc::RUNTIME>(P, S, lane, npairs, cnt);
         __syncwarp();
     }
     if (STATS) cnt.flush(P.ws);

@@ -336,8 +336,8 @@ template <bool STATS, int MINB, Acc A, int PASS>
 __global__ void __launch_bounds__(128, MINB) k_oct_warp(const DepositParams P)
 {
     constexpr bool FIRST = PASS == kPassFp32;
+    using T = typename PassScalar<PASS>::type;
     WarpSmem *S = warp_smem(!FIRST);
-    bind_residuals(P, S, !FIRST);
     const int lane = threadIdx.x & 31;
     Counters cnt;
     if (STATS) cnt.zero();
@@ -384,6 +384,7 @@ __global__ void __launch_bounds__(128, MINB) k_oct_warp(const DepositParams P)
                 if (!have) set_error(P.ws, 3, (int)(u & 0x7fffffff));
             }
         }
+#pragma unroll 1
         for (int si = 0; si < (LIST ? 1 : 6); ++si) {
             const int s = LIST ? s_listed : si;
             bool to_list = false;  // the FP32 pass: a pair of this tetrahedron is guarded
@@ -439,23 +440,22 @@ __global__ void __launch_bounds__(128, MINB) k_oct_warp(const DepositParams P)
                             set_error(P.ws, 4, lane);
                             more = false;
                         } else {
-                            int lo[3], dim[3];
+                            int lo[3], dim[3], org[3];
 #pragma unroll
                             for (int a = 0; a < 3; ++a) {
-                                const int org = (int)(hit.org[a] - base[a]);
-                                lo[a] = ts.lo[a] > org ? ts.lo[a] : org;
-                                const int hi = ts.lo[a] + ts.dim[a] - 1 < org + (int)bc - 1 ? ts.lo[a] + ts.dim[a] - 1
-                                                                                            : org + (int)bc - 1;
+                                org[a] = (int)(hit.org[a] - base[a]);
+                                lo[a] = ts.lo[a] > org[a] ? ts.lo[a] : org[a];
+                                const int top = org[a] + (int)bc - 1;
+                                const int hi = ts.lo[a] + ts.dim[a] - 1 < top ? ts.lo[a] + ts.dim[a] - 1 : top;
                                 dim[a] = hi - lo[a] + 1;
-                                S->org[a][lane] = org;
                             }
                             const int64_t ncell = (int64_t)dim[0] * dim[1] * dim[2];
                             if (!FIRST && (single || !guard)) {
                                 // the guarded pass: nothing to do for this pair
                             } else if (single) {
                                 // whole tetrahedron inside one cell of this leaf
-                                cell_add<A>(P, P.out + (int64_t)hit.leaf * bc * bc * bc + (lo[0] - S->org[0][lane]) +
-                                              bc * ((lo[1] - S->org[1][lane]) + bc * (lo[2] - S->org[2][lane])),
+                                cell_add<A>(P, P.out + (int64_t)hit.leaf * bc * bc * bc + (lo[0] - org[0]) +
+                                              bc * ((lo[1] - org[1]) + bc * (lo[2] - org[2])),
                                           m_t);
                                 cnt.add_dep(m_t);
                                 if (STATS) { cnt.u[ST_SINGLE_CELL]++; cnt.u[ST_BBOX_CELLS]++; cnt.u[ST_OVERLAPPED]++; }
@@ -471,44 +471,15 @@ __global__ void __launch_bounds__(128, MINB) k_oct_warp(const DepositParams P)
                                     cnt.u[ST_BBOX_CELLS] += ncell;
                                     cnt.u[ST_BIN0 + size_bin(ncell)]++;
                                 }
-#pragma unroll
-                                for (int q = 0; q < 4; ++q) {
-                                    S->v[3 * q][lane] = ts.v[q].x;
-                                    S->v[3 * q + 1][lane] = ts.v[q].y;
-                                    S->v[3 * q + 2][lane] = ts.v[q].z;
-                                    S->n[3 * q][lane] = ts.n[q].x;
-                                    S->n[3 * q + 1][lane] = ts.n[q].y;
-                                    S->n[3 * q + 2][lane] = ts.n[q].z;
-                                    S->e[q][lane] = ts.e[q];
-                                    S->pos[q][lane] = ts.pos[q];
-                                    S->neg[q][lane] = ts.neg[q];
-                                }
-#pragma unroll
-                                for (int a = 0; a < 3; ++a) {
-                                    S->lo[a][lane] = lo[a];
-                                    S->dim[a][lane] = dim[a];
-                                    S->base[a][lane] = base[a];
-                                }
                                 S->leaf[lane] = hit.leaf;
-                                bool flip = false;
-                                S->rho[lane] = guard ? (float)(6.0 * m_t / exact_vol6(ts.v, res, ts.vol6, &flip))
-                                                     : __fdiv_rn((float)(6.0 * m_t), (float)ts.vol6);
-                                S->lx[lane] = ts.lx;
-                                S->ly[lane] = ts.ly;
-                                S->axis[lane] = ts.axis;
-                                S->guard[lane] = guard ? (1 | (flip ? kGuardFlip : 0)) : 0;
-                                S->skip[lane] = 0;
-                                {
-                                    const int C = ts.axis;
-                                    S->cut[lane] = (C == 0 ? lo[0] > ts.lo[0] : (C == 1 ? lo[1] > ts.lo[1] : lo[2] > ts.lo[2]))
-                                                       ? 1 : 0;
-                                }
-                                if (guard) store_residuals(S, lane, res);
+                                const int C = ts.axis;
+                                const bool cut = C == 0 ? lo[0] > ts.lo[0] : (C == 1 ? lo[1] > ts.lo[1] : lo[2] > ts.lo[2]);
+                                store_record<PASS>(S, lane, ts, res, lo, dim, org, m_t, P.kappa_max, cut);
                             }
                         }
                     }
                 }
-                coop_pairs<STATS, true, A, PASS>(P, S, lane, npairs, cnt);
+                coop_runs<STATS, true, A, T>(P, S, lane, npairs, 0, cnt);
                 __syncwarp();
             }
             __syncwarp();
