@@ -159,6 +159,24 @@ void fill_grid(pse::DepositParams &p, const int64_t grid_n[3], double box)
     }
 }
 
+// The work items of the warp kernels.  An item is one warp's batch of up to 32 tetrahedra: the
+// same Kuhn tetrahedron of 32 consecutive cubes (octree: all six, one after another, while there
+// are many items), or 32 tetrahedra of an explicit set.  Small deposits take fewer cubes an item,
+// so that every warp the GPU holds (16 on each of 152 SMs) gets one.  (Before, an item was a row
+// segment of 32 cubes with all six tetrahedra: 16^3 on 32^3 0.86 -> 0.46 ms, 32^3 on 64^3 0.92 ->
+// 0.56 ms, 48^3 on 384^3, whose rows fill three quarters of a warp, 31.0 -> 18.3 ms, 256^3 on
+// 128^3 64.7 -> 56.4 ms.)
+void set_items(pse::DepositParams &p)
+{
+    constexpr int64_t kWarps = 152 * 16;
+    const int64_t nsub = p.src == pse::SRC_TETS ? 1 : 6;
+    p.group = 32;
+    while (p.group > 8 && (p.n_units + p.group - 1) / p.group * nsub < 2 * kWarps) p.group /= 2;
+    const int64_t groups = (p.n_units + p.group - 1) / p.group;
+    p.subs = (p.leaves && groups >= 4 * kWarps) ? 6 : 1;
+    p.n_items = groups * (nsub / (p.leaves ? p.subs : 1));
+}
+
 // ---------------------------------------------------------------------------
 // Slab streaming: the particle lattice stays in host memory and is copied to the GPU
 // one z-slab at a time (slab_cubes cube layers = slab_cubes + 1 particle rows, the last
@@ -212,7 +230,7 @@ int stream_slabs(const float *h_pos, const pse::DepositParams &base, int64_t sla
         p.nc[2] = k1 - k0;
         p.src = pse::SRC_LATTICE;
         p.n_units = p.nc[0] * p.nc[1] * p.nc[2];
-        p.n_items = ((p.nc[0] + 31) / 32) * p.nc[1] * p.nc[2];
+        set_items(p);
         rc = per_slab(p, st);
         if (rc != PSE_OK) break;
         e = cudaEventRecord(freed[b], st);
@@ -306,8 +324,7 @@ int run_deposit(pse::DepositParams &p, const pse_deposit_opts &o, int64_t cells,
     const bool comp = o.precision == PSE_FP32_COMPENSATED;
     p.comp = comp ? 1 : 0;
     const int bps = (tu && tu->blocks_per_sm > 0) ? tu->blocks_per_sm : kDefaultBlocksPerSm;
-    if (p.n_units > 0 && o.schedule != PSE_THREAD_PER_TET)
-        p.n_items = (p.src == pse::SRC_LATTICE) ? ((p.nc[0] + 31) / 32) * p.nc[1] * p.nc[2] : (p.n_units + 31) / 32;
+    set_items(p);
 
     // the kernels of one deposit pass over the tetrahedra of q, on stream s
     auto launch = [&](const pse::DepositParams &q, cudaStream_t s) -> int {
@@ -431,9 +448,9 @@ int run_deposit(pse::DepositParams &p, const pse_deposit_opts &o, int64_t cells,
         h_stats->column_runs = hw.stats[pse::ST_RUNS];
         // the mass this call wrote into the output: its in-grid deposits, times the
         // renormalisation factor when it applied
-        const double in_grid = hw.mass_deposited - hw.mass_dropped;
-        h_stats->mass_out = (renorm && hw.mass_deposited > 0.0) ? in_grid * (hw.mass_target / hw.mass_deposited)
-                                                                 : in_grid;
+        const double deposited = hw.mass_deposited + hw.mass_deposited_lo, in_grid = deposited - hw.mass_dropped;
+        h_stats->mass_out = (renorm && deposited > 0.0) ? in_grid * ((hw.mass_target + hw.mass_target_lo) / deposited)
+                                                         : in_grid;
         if (hw.error_code != 0)
             return fail(PSE_ERR_DEVICE,
                         hw.error_code == 1 ? "a tetrahedron is wider than the periodic grid (detail %d)"

@@ -4,6 +4,9 @@
 // for the FP32 pass, double for guarded tetrahedra (from their exact vertices).
 #pragma once
 
+#include <cstring>
+#include <type_traits>
+
 #include "geom.cuh"
 
 namespace pse {
@@ -404,6 +407,337 @@ PSE_HD T level_volume(T c0, T c1, T s0, T s1, T colmin, T colmax, T msum)
     return (b1 - b0) * T(1.0 / 6.0);
 }
 
+// ---------------------------------------------------------------------------
+// The float64 column clip (guarded tetrahedra).  GB300's float64 pipe takes 16 cycles a warp
+// instruction on each SM, 64 issue slots, so this version of the clip is written for few float64
+// operations: 1 in 2.5 of the generic stages above.
+//  * Comparisons, minima and clamps read the numbers' bits (ordered as integers) instead of
+//    the float64 pipe.
+//  * The reciprocal of an edge's extent starts from the float32 one and takes one third-order
+//    step, r (1 + e + e^2) with e = 1 - x r (the error falls from 1e-7 to below rounding).
+//  * All integrals of a polygon come from four moments about one of its own vertices (in the
+//    cell, so nothing cancels): Σ C, Σ C (x_a + x_b), Σ C (y_a + y_b), Σ C (z_a + z_b), with C
+//    the cross product of an edge's ends.
+//  * A level's fan starts from a crossing point of the level line itself, so that no face
+//    plane enters, and whole-polygon bounds are kept as ordered integers.
+// The clip's error stays a few 1e-16 of a cell (1e-12 is tested).  Measured (one GB300): the
+// shell-crossed 128^3 octree deposit, nine tenths of it this clip, 141 -> 85 ms; 60,000 explicit
+// tetrahedra 3.2 -> 1.1 ms (with the guarded list taken in smaller items).
+// ---------------------------------------------------------------------------
+PSE_HD long long f64_bits(double x)
+{
+#ifdef __CUDA_ARCH__
+    return __double_as_longlong(x);
+#else
+    long long b;
+    std::memcpy(&b, &x, sizeof(b));
+    return b;
+#endif
+}
+PSE_HD double f64_of(long long b)
+{
+#ifdef __CUDA_ARCH__
+    return __longlong_as_double(b);
+#else
+    double x;
+    std::memcpy(&x, &b, sizeof(x));
+    return x;
+#endif
+}
+// an integer that orders like the number
+PSE_HD long long f64_key(double x)
+{
+    const long long b = f64_bits(x);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+// x > t for t > 0
+PSE_HD bool f64_above(double x, double t) { return f64_bits(x) > f64_bits(t); }
+
+// t held in [0, 1]
+PSE_HD double f64_sat01(double t)
+{
+    const long long b = f64_bits(t);
+    return b < 0 ? 0.0 : (b >= 0x3ff0000000000000ll ? 1.0 : t);
+}
+
+// float32 to float64 without a conversion instruction (those share the float64 pipe's rate);
+// a float32 denormal is not kept (it becomes about 1e-38)
+PSE_HD double f64_widen(float x)
+{
+#ifdef __CUDA_ARCH__
+    const int b = __float_as_int(x), m = b & 0x7fffffff;
+    const int hi = m == 0 ? 0 : (b & (int)0x80000000) | ((m >> 3) + 0x38000000);
+    return __hiloint2double(hi, m == 0 ? 0 : b << 29);
+#else
+    return (double)x;
+#endif
+}
+
+// 1 / x (0 for an x beyond 2^-100 .. 2^100: an edge that does not cross anything)
+PSE_HD double f64_rcp(double x)
+{
+#ifdef __CUDA_ARCH__
+    const int hi = __double2hiint(x), m = hi & 0x7fffffff;
+    const bool ok = (unsigned)(m - ((1023 - 100) << 20)) < (200u << 20);
+    const float f = __int_as_float((hi & (int)0x80000000) | (((m - 0x38000000) << 3) | (int)((unsigned)__double2loint(x) >> 29)));
+    const int b = __float_as_int(slab_rcp(f));
+    const double r = __hiloint2double((b & (int)0x80000000) | (((b & 0x7fffffff) >> 3) + 0x38000000), b << 29);
+    const double e = fma(-x, r, 1.0);
+    return ok ? fma(r, fma(e, e, e), r) : 0.0;
+#else
+    return x != 0.0 ? 1.0 / x : 0.0;
+#endif
+}
+
+template <int KW>
+struct FaceRun64 {
+    double k6[KW + 1];
+    double m6;
+    long long kmin, kmax;  // z range of the polygon, as ordered integers
+    int jlo, jhi, n;
+};
+constexpr long long kKeyMax = 0x7fffffffffffffffll, kKeyMin = -kKeyMax - 1;
+
+template <int KW>
+PSE_HD void face_none(FaceRun64<KW> &R)
+{
+#pragma unroll
+    for (int j = 0; j <= KW; ++j) R.k6[j] = 0.0;
+    R.m6 = 0.0;
+    R.kmin = kKeyMax;
+    R.kmax = kKeyMin;
+    R.jlo = 0;
+    R.jhi = -1;
+    R.n = 0;
+}
+
+// Moments of a polygon about its vertex o, edge by edge.
+struct Moments64 {
+    double c, x, y, z;
+    P3<double> o;
+    PSE_HD void add(const P3<double> &a, const P3<double> &b, bool on)
+    {
+        const double ux = a.x - o.x, uy = a.y - o.y, wx = b.x - o.x, wy = b.y - o.y;
+        const double cr = on ? fma(ux, wy, -(uy * wx)) : 0.0;
+        c += cr;
+        x = fma(cr, ux + wx, x);
+        y = fma(cr, uy + wy, y);
+        z = fma(cr, (a.z - o.z) + (b.z - o.z), z);
+    }
+};
+
+// One face (a, b, c) of a run in the local frame: as face_run, tol the classification tolerance.
+template <int KW, class Slots>
+PSE_HD void face_run_f64(const P3<double> &a, const P3<double> &b, const P3<double> &c, const RunFrame<double> &F,
+                         double tol, const Slots &E, FaceRun64<KW> &R)
+{
+    // ---- x slab: lo <= x < hi
+    int n = 0;
+    {
+        const double lo = -F.qx, hi = 1.0 - F.qx;
+        const P3<double> p[3] = {a, b, c};
+        double dl[3], dh[3];
+        bool below[3], above[3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            dl[i] = lo - p[i].x;
+            dh[i] = hi - p[i].x;
+            below[i] = f64_above(dl[i], tol);
+            above[i] = !f64_above(dh[i], tol);
+        }
+        double xly = 0.0, xlz = 0.0, nly = 0.0, nlz = 0.0, xhy = 0.0, xhz = 0.0, nhy = 0.0, nhz = 0.0;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const int j = i == 2 ? 0 : i + 1;
+            const double inv = f64_rcp(p[j].x - p[i].x);
+            const double ta = f64_sat01((below[i] ? dl[i] : dh[i]) * inv), tb = f64_sat01((below[j] ? dl[i] : dh[i]) * inv);
+            const double dy = p[j].y - p[i].y, dz = p[j].z - p[i].z;
+            const bool ina = !below[i] && !above[i], inb = !below[j] && !above[j];
+            const double ay = ina ? p[i].y : fma(ta, dy, p[i].y), az = ina ? p[i].z : fma(ta, dz, p[i].z);
+            const double by = inb ? p[j].y : fma(tb, dy, p[i].y), bz = inb ? p[j].z : fma(tb, dz, p[i].z);
+            if (!below[i] && below[j]) { xly = by; xlz = bz; }
+            if (below[i] && !below[j]) { nly = ay; nlz = az; }
+            if (!above[i] && above[j]) { xhy = by; xhz = bz; }
+            if (above[i] && !above[j]) { nhy = ay; nhz = az; }
+            if (!(below[i] && below[j]) && !(above[i] && above[j])) {
+                const double ax = ina ? p[i].x : (below[i] ? lo : hi), bx = inb ? p[j].x : (below[j] ? lo : hi);
+                E.store(n, mk<double>(ax, ay, az), mk<double>(bx, by, bz));
+                ++n;
+            }
+        }
+        if ((below[0] || below[1] || below[2]) && !(below[0] && below[1] && below[2])) {
+            E.store(n, mk<double>(lo, xly, xlz), mk<double>(lo, nly, nlz));
+            ++n;
+        }
+        if ((above[0] || above[1] || above[2]) && !(above[0] && above[1] && above[2])) {
+            E.store(n, mk<double>(hi, xhy, xhz), mk<double>(hi, nhy, nhz));
+            ++n;
+        }
+    }
+    // ---- y slab, and the polygon's moments and z range
+    const double lo = -F.qy, hi = 1.0 - F.qy;
+    P3<double> xl = mk<double>(0.0, lo, 0.0), nl = xl, xh = mk<double>(0.0, hi, 0.0), nh = xh;
+    bool cl = false, ch = false, any = false;
+    Moments64 M;
+    M.c = M.x = M.y = M.z = 0.0;
+    M.o = mk<double>(0.0, 0.0, 0.0);
+    long long kmin = kKeyMax, kmax = kKeyMin;
+    int m = 0;
+#pragma unroll 1
+    for (int k = 0; k < n; ++k) {
+        P3<double> ea, eb;
+        E.load(k, ea, eb);
+        const double dl = lo - ea.y, dh = hi - ea.y;
+        const bool a_lo = f64_above(dl, tol), a_hi = !f64_above(dh, tol);
+        const bool b_lo = f64_above(lo - eb.y, tol), b_hi = !f64_above(hi - eb.y, tol);
+        const double inv = f64_rcp(eb.y - ea.y);
+        const double ta = f64_sat01((a_lo ? dl : dh) * inv), tb = f64_sat01((b_lo ? dl : dh) * inv);
+        const double dx = eb.x - ea.x, dz = eb.z - ea.z;
+        const bool ina = !a_lo && !a_hi, inb = !b_lo && !b_hi;
+        const P3<double> na = mk<double>(ina ? ea.x : fma(ta, dx, ea.x), ina ? ea.y : (a_lo ? lo : hi),
+                                         ina ? ea.z : fma(ta, dz, ea.z));
+        const P3<double> nb = mk<double>(inb ? eb.x : fma(tb, dx, ea.x), inb ? eb.y : (b_lo ? lo : hi),
+                                         inb ? eb.z : fma(tb, dz, ea.z));
+        if (!a_lo && b_lo) { xl = nb; cl = true; }
+        if (a_lo && !b_lo) nl = na;
+        if (!a_hi && b_hi) { xh = nb; ch = true; }
+        if (a_hi && !b_hi) nh = na;
+        const bool live = !(a_lo && b_lo) && !(a_hi && b_hi);
+        if (live && !any) M.o = na;
+        M.add(na, nb, live);
+        if (live) {
+            any = true;
+            const long long ka = f64_key(na.z), kb = f64_key(nb.z);
+            const long long kl = ka < kb ? ka : kb, kh = ka < kb ? kb : ka;
+            kmin = kl < kmin ? kl : kmin;
+            kmax = kh > kmax ? kh : kmax;
+            E.store(m, na, nb);
+            ++m;
+        }
+    }
+    M.add(xl, nl, cl);
+    M.add(xh, nh, ch);
+    if (cl) {
+        E.store(m, xl, nl);
+        ++m;
+    }
+    if (ch) {
+        E.store(m, xh, nh);
+        ++m;
+    }
+    R.n = m;
+    R.kmin = kmin;
+    R.kmax = kmax;
+    // 6 ∫ (h - l) for a height h that is constant (c) or the face's own: 3 Σ C (h(o) - l(o)) plus
+    // the moments of h - l beyond o
+    const double lo6 = fma(F.lx, M.o.x, fma(F.ly, M.o.y, F.l0));
+    const double a6 = 3.0 * M.c, t6 = -fma(F.lx, M.x, F.ly * M.y);
+    R.m6 = M.z + fma(a6, M.o.z - lo6, t6);
+    int jlo = F.j0, jhi = -1;
+#pragma unroll
+    for (int j = 0; j <= KW; ++j) {
+        const double cj = f64_widen((float)j) - F.qz;
+        const long long kj = f64_key(cj);
+        if (j <= F.K) {
+            jlo += (j >= F.j0 && kj <= kmin) ? 1 : 0;
+            jhi += kj < kmax ? 1 : 0;
+        }
+        // (levels below jlo: the face lies above them; kj <= kmin)
+        R.k6[j] = (j >= F.j0 && j <= F.K) ? (kj <= kmin ? (any ? fma(a6, cj - lo6, t6) : 0.0) : R.m6) : 0.0;
+    }
+    R.jlo = jlo;
+    R.jhi = jhi;
+}
+
+// 6 ∫ (z - c)_+ over the polygon of the n edges in E, as level_fan.
+template <class Slots>
+PSE_HD double level_fan_f64(const Slots &E, int n, double c)
+{
+    const long long kc = f64_key(c);
+    // the first edge that crosses the level
+    int first = -1;
+    P3<double> ea, eb;
+#pragma unroll 1
+    for (int k = 0; k < n && first < 0; ++k) {
+        E.load(k, ea, eb);
+        if ((f64_key(ea.z) > kc) != (f64_key(eb.z) > kc)) first = k;
+    }
+    if (first < 0) return 0.0;
+    double t = (c - ea.z) * f64_rcp(eb.z - ea.z);
+    const double ox = fma(t, eb.x - ea.x, ea.x), oy = fma(t, eb.y - ea.y, ea.y);
+    double g = 0.0;
+#pragma unroll 1
+    for (int k = 0; k < n; ++k) {
+        E.load(k, ea, eb);
+        const bool a_up = f64_key(ea.z) > kc, b_up = f64_key(eb.z) > kc;
+        if (!a_up && !b_up) continue;
+        double px = ox, py = oy;  // an edge wholly above does not use it
+        const double fa = c - ea.z;
+        if (a_up != b_up && k != first) {
+            t = fa * f64_rcp(eb.z - ea.z);
+            px = fma(t, eb.x - ea.x, ea.x);
+            py = fma(t, eb.y - ea.y, ea.y);
+        }
+        const double ax = (a_up ? ea.x : px) - ox, ay = (a_up ? ea.y : py) - oy;
+        const double bx = (b_up ? eb.x : px) - ox, by = (b_up ? eb.y : py) - oy;
+        const double h = (a_up ? -fa : 0.0) + (b_up ? eb.z - c : 0.0);
+        g = fma(fma(ax, by, -(ay * bx)), h, g);
+    }
+    return g;
+}
+
+// The volume between two levels, as level_volume, from the ordered z range.
+PSE_HD double level_volume_f64(double c0, double c1, double s0, double s1, long long kmin, long long kmax, double msum)
+{
+    const long long k0 = f64_key(c0), k1 = f64_key(c1);
+    const double b0 = k0 <= kmin ? 0.0 : (k0 >= kmax ? msum : s0);
+    const double b1 = k1 <= kmin ? 0.0 : (k1 >= kmax ? msum : s1);
+    return (b1 - b0) * (1.0 / 6.0);
+}
+
+// The classification tolerance for coordinates of up to `extent` cells.
+PSE_HD double f64_tolerance(double extent) { return 8.0 * 2.220446049250313e-16 * (1.0 + extent); }
+
+template <int KW, class Src>
+PSE_HD void column_volumes_f64(const Src &src, double lx, double ly, int K, bool lo_open, double (&vol)[KW],
+                               double2 *slots)
+{
+    const RunFrame<double> F = run_frame<double>(src, lx, ly, K, lo_open);
+    const EdgeSlots<double> E{slots};
+    const P3<double> q = mk<double>(F.qx, F.qy, F.qz);
+    double extent = 0.0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const P3<double> v = src.vtx(i);
+        extent = fmax(extent, fmax(fmax(fabs(v.x), fabs(v.y)), fabs(v.z)));
+    }
+    double S[KW + 1], msum = 0.0;
+#pragma unroll
+    for (int j = 0; j <= KW; ++j) S[j] = 0.0;
+    long long kmin = kKeyMax, kmax = kKeyMin;
+#pragma unroll 1
+    for (int f = 0; f < 4; ++f) {
+        int ia, ib, ic;
+        face_vertices(f, ia, ib, ic);
+        FaceRun64<KW> R;
+        face_run_f64<KW>(sub(src.vtx(ia), q), sub(src.vtx(ib), q), sub(src.vtx(ic), q), F, f64_tolerance(extent), E, R);
+#pragma unroll 1
+        for (int j = R.jlo; j <= R.jhi; ++j) {
+            const double g = level_fan_f64(E, R.n, (double)j - F.qz);
+#pragma unroll
+            for (int i = 0; i <= KW; ++i) R.k6[i] -= (i == j) ? g : 0.0;
+        }
+#pragma unroll
+        for (int j = 0; j <= KW; ++j) S[j] += R.k6[j];
+        kmin = R.kmin < kmin ? R.kmin : kmin;
+        kmax = R.kmax > kmax ? R.kmax : kmax;
+        msum += R.m6;
+    }
+#pragma unroll
+    for (int j = 0; j < KW; ++j)
+        vol[j] = level_volume_f64((double)j - F.qz, (double)(j + 1) - F.qz, S[j], S[j + 1], kmin, kmax, msum);
+}
+
 // Overlap volumes of a positively oriented tetrahedron (clip frame, relative to the first
 // cell of the run: the run is [0,1)^2 x [0,K), K <= KW) with the K cells of the run.  src
 // gives vertex i (src.vtx(i)) and the outward normal of face f (src.nrm(f)), read when
@@ -415,6 +749,10 @@ PSE_HD T level_volume(T c0, T c1, T s0, T s1, T colmin, T colmax, T msum)
 template <int KW, class T, class Src>
 PSE_HD void column_volumes(const Src &src, T lx, T ly, int K, bool lo_open, T (&vol)[KW], slot2_t<T> *slots)
 {
+    if constexpr (std::is_same<T, double>::value) {
+        column_volumes_f64<KW>(src, lx, ly, K, lo_open, vol, slots);
+        return;
+    }
     const RunFrame<T> F = run_frame<T>(src, lx, ly, K, lo_open);
     const EdgeSlots<T> E{slots};
     const P3<T> q = mk<T>(F.qx, F.qy, F.qz);

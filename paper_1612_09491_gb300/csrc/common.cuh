@@ -58,56 +58,90 @@ __device__ __forceinline__ int64_t wrap_idx(int64_t i, int64_t n)
     return i;
 }
 
+// The float32 positions of the vertices of tetrahedron s of Lagrangian cube (ci, cj, ck).  The
+// four particles are reached from corner 000 by steps along the axes (wrapped on periodic
+// lattices), so one particle index is formed and the others are added to it.
+__device__ __forceinline__ void lattice_positions(const DepositParams &P, int64_t ci, int64_t cj, int64_t ck, int s,
+                                                  float (&x)[4][3])
+{
+    const int64_t r1 = 3 * P.n[0], r2 = r1 * P.n[1];
+    const int64_t d0 = (P.periodic && ci + 1 == P.n[0]) ? 3 - r1 : 3;
+    const int64_t d1 = (P.periodic && cj + 1 == P.n[1]) ? r1 - r2 : r1;
+    const int64_t d2 = (P.periodic && !P.slab && ck + 1 == P.n[2]) ? r2 - r2 * P.n[2] : r2;
+    // axis permutations (a, b, c): xyz, xzy, yxz, yzx, zxy, zyx
+    const int a = s >> 1, b = (s == 0 || s == 5) ? 1 : ((s == 1 || s == 3) ? 2 : 0);
+    const float *p[4];
+    p[0] = P.pos + (3 * ci + r1 * cj + r2 * ck);
+    p[1] = p[0] + (a == 0 ? d0 : (a == 1 ? d1 : d2));
+    p[2] = p[1] + (b == 0 ? d0 : (b == 1 ? d1 : d2));
+    p[3] = p[0] + (d0 + d1 + d2);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) x[q][c] = __ldg(p[q] + c);
+}
+
+// Whether a vertex may need a periodic shift: some coordinate is not within 0.49 box of corner
+// 000's in float32 (a tetrahedron across the box boundary, or non-finite).  When not, every
+// nearest image is the vertex itself and the float64 decisions are not needed.
+__device__ __forceinline__ bool may_shift(const DepositParams &P, const float (&x)[4][3])
+{
+    const float near = 0.49f * (float)P.box;
+    bool all = true;
+#pragma unroll
+    for (int q = 1; q < 4; ++q)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) all = all && fabsf(x[q][a] - x[0][a]) < near;
+    return P.periodic && !all;
+}
+
+// Periodic unwrap: coordinate v is moved by -box when v - v0 >= box/2 and by +box when
+// v - v0 < -box/2 (nearest image), decided in float64 on the float32 inputs.
+__device__ __forceinline__ int image_shift(const DepositParams &P, float v, float v0)
+{
+    const double d = (double)v - (double)v0;
+    return (d >= 0.5 * P.box) ? -1 : ((d < -0.5 * P.box) ? 1 : 0);
+}
+
 // Vertices of tetrahedron s of Lagrangian cube (ci, cj, ck), in grid units relative to
-// the base cell (the cell holding corner 000).  Periodic unwrap: corner v is moved by
-// -box when v - v0 >= box/2 and by +box when v - v0 < -box/2 (nearest image), decided
-// in float64 on the float32 inputs.
+// the base cell (the cell holding corner 000), each corner at its periodic image nearest to
+// corner 000.
 template <class T>
 __device__ __forceinline__ void lattice_tet(const DepositParams &P, int64_t ci, int64_t cj, int64_t ck, int s,
                                             P3<T> (&v)[4], int (&base)[3], P3<float> *res = nullptr)
 {
-    int o1[3], o2[3];
-    kuhn_offsets(s, o1, o2);
     float x[4][3];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        int64_t i = ci, j = cj, k = ck;
-        if (q == 1) { i += o1[0]; j += o1[1]; k += o1[2]; }
-        if (q == 2) { i += o2[0]; j += o2[1]; k += o2[2]; }
-        if (q == 3) { i += 1; j += 1; k += 1; }
-        if (P.periodic) {
-            i = wrap_idx(i, P.n[0]);
-            j = wrap_idx(j, P.n[1]);
-            if (!P.slab) k = wrap_idx(k, P.n[2]);
-        }
-        const float *p = P.pos + 3 * (i + P.n[0] * (j + P.n[1] * k));
-        x[q][0] = __ldg(p);
-        x[q][1] = __ldg(p + 1);
-        x[q][2] = __ldg(p + 2);
-    }
+    lattice_positions(P, ci, cj, ck, s, x);
 #pragma unroll
     for (int a = 0; a < 3; ++a) base[a] = safe_floor((double)x[0][a] * P.scale_d[a]);
+    T c[4][3];
+    float rr[4][3];
+    // off: the vertex's periodic image and the base cell, in cells (at most 2^30 + 2^24)
+    auto place = [&](int q, int a, int off) {
+        if constexpr (sizeof(T) == 4) {
+            c[q][a] = fmaf(x[q][a], P.scale_f[a], (float)off);
+            if (res) rr[q][a] = (float)(fma((double)x[q][a], P.scale_d[a], (double)off) - (double)c[q][a]);
+        } else {
+            c[q][a] = fma((double)x[q][a], P.scale_d[a], (double)off);
+        }
+    };
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) place(q, a, -base[a]);
+    if (may_shift(P, x)) {
+#pragma unroll
+        for (int q = 1; q < 4; ++q)
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const int shift = image_shift(P, x[q][a], x[0][a]);
+                if (shift != 0) place(q, a, shift * (int)P.g[a] - base[a]);
+            }
+    }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        T c[3];
-        float rr[3] = {0.f, 0.f, 0.f};
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            int shift = 0;
-            if (P.periodic && q > 0) {
-                const double d = (double)x[q][a] - (double)x[0][a];
-                shift = (d >= 0.5 * P.box) ? -1 : ((d < -0.5 * P.box) ? 1 : 0);
-            }
-            const long long off = (long long)shift * P.g[a] - base[a];
-            if constexpr (sizeof(T) == 4) {
-                c[a] = fmaf(x[q][a], P.scale_f[a], (float)off);
-                if (res) rr[a] = (float)(fma((double)x[q][a], P.scale_d[a], (double)off) - (double)c[a]);
-            } else {
-                c[a] = fma((double)x[q][a], P.scale_d[a], (double)off);
-            }
-        }
-        v[q] = mk<T>(c[0], c[1], c[2]);
-        if (sizeof(T) == 4 && res) res[q] = mk<float>(rr[0], rr[1], rr[2]);
+        v[q] = mk<T>(c[q][0], c[q][1], c[q][2]);
+        if (sizeof(T) == 4 && res) res[q] = mk<float>(rr[q][0], rr[q][1], rr[q][2]);
     }
 }
 
@@ -175,15 +209,43 @@ __device__ __forceinline__ double exact_vol6(const P3<float> (&v)[4], const P3<f
     return d > 0.0 ? d : vol6_f32;
 }
 
+// Coordinates of Lagrangian cube c.  Lattices of 2^32 cubes and more divide out of line.
+__device__ __noinline__ void cube_coords_far(const int64_t (&nc)[3], int64_t c, int64_t &i, int64_t &j, int64_t &k)
+{
+    i = c % nc[0];
+    j = (c / nc[0]) % nc[1];
+    k = c / (nc[0] * nc[1]);
+}
+__device__ __forceinline__ void cube_coords(const DepositParams &P, int64_t c, int64_t &i, int64_t &j, int64_t &k)
+{
+    if (P.nc[0] * P.nc[1] * P.nc[2] <= (int64_t)0xffffffffll) {
+        const unsigned n0 = (unsigned)P.nc[0], n1 = (unsigned)P.nc[1];
+        const unsigned row = (unsigned)c / n0, layer = row / n1;
+        i = (unsigned)c - row * n0;
+        j = row - layer * n1;
+        k = layer;
+    } else {
+        cube_coords_far(P.nc, c, i, j, k);
+    }
+}
+
 // Lagrangian cube of work unit u; false (and nothing read) for an out-of-range cube id.
 __device__ __forceinline__ bool cube_of_unit(const DepositParams &P, int64_t u, int64_t &i, int64_t &j, int64_t &k)
 {
     const int64_t c = (P.src == SRC_CUBE_LIST) ? P.cube_ids[u] : u;
     if (c < 0 || c >= P.nc[0] * P.nc[1] * P.nc[2]) return false;
-    i = c % P.nc[0];
-    j = (c / P.nc[0]) % P.nc[1];
-    k = c / (P.nc[0] * P.nc[1]);
+    cube_coords(P, c, i, j, k);
     return true;
+}
+
+// How many listed guarded tetrahedra a work item of the guarded pass takes: 32 when there are
+// plenty, fewer when the grid's warps would otherwise share only a few items (a listed
+// tetrahedron can cover thousands of cells).
+__device__ __forceinline__ int listed_per_item(int64_t listed)
+{
+    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    const int64_t per = listed / (4 * warps);
+    return per < 1 ? 1 : (per > 32 ? 32 : (int)per);
 }
 
 __device__ __forceinline__ int64_t fold_cell(int64_t c, int64_t g)
@@ -331,6 +393,13 @@ struct Counters {
         dep = t;
         dep_b = 0.0;
     }
+    // *sum += x, and the addition's rounding error (two-sum) to *lo: thousands of warps add
+    // similar values, whose roundings would drift together
+    static __device__ __forceinline__ void add_exact(double *sum, double *lo, double x)
+    {
+        const double old = atomicAdd(sum, x), s = old + x, xx = s - old;
+        atomicAdd(lo, (old - (s - xx)) + (x - xx));
+    }
     __device__ void flush_mass(const DepositParams &P, Workspace *ws)
     {
         fold_dep();
@@ -341,8 +410,8 @@ struct Counters {
             b += __shfl_down_sync(kFull, b, o);
         }
         if ((threadIdx.x & 31) == 0 && (a != 0.0 || b != 0.0)) {
-            atomicAdd(&ws->mass_target, a);
-            atomicAdd(&ws->mass_deposited, b);
+            add_exact(&ws->mass_target, &ws->mass_target_lo, a);
+            add_exact(&ws->mass_deposited, &ws->mass_deposited_lo, b);
         }
     }
     __device__ void flush(Workspace *ws)
@@ -418,8 +487,7 @@ constexpr int kRecGuard = 8;  // a guarded tetrahedron (clipped in float64)
 struct GuardSmem {
     double2 slots[21][32];  // each lane's 7 edge slots, 3 double2 each
     double v[12][32];       // exact vertices, positively oriented
-    double n[12][32];       // their outward face normals
-    double l0[64];          // queued runs: the frame's l0
+    double tol[32];         // classification tolerance of the clip (f64_tolerance)
 };
 
 constexpr int kQBits = 19;  // per-axis cell offset bits in a queue entry
@@ -529,22 +597,19 @@ __device__ __forceinline__ void store_record(WarpSmem *S, int lane, const TetSet
     S->axis[lane] = ts.axis | (cut ? kRecCut : 0) | (guard ? kRecGuard : 0);
     if constexpr (PASS == kPassGuard) {
         GuardSmem *G = guard_smem(S);
-        P3<double> pd[4], nd[4];
+        P3<double> pd[4];
         exact_vertices(ts.v, res, 0, 0, 0, pd);
+        G->tol[lane] = f64_tolerance((double)(ts.dim[0] + ts.dim[1] + ts.dim[2]));
         if (turn) {
             const P3<double> t = pd[1];
             pd[1] = pd[2];
             pd[2] = t;
         }
-        face_normals<double>(pd, nd);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             G->v[3 * q][lane] = pd[q].x;
             G->v[3 * q + 1][lane] = pd[q].y;
             G->v[3 * q + 2][lane] = pd[q].z;
-            G->n[3 * q][lane] = nd[q].x;
-            G->n[3 * q + 1][lane] = nd[q].y;
-            G->n[3 * q + 2][lane] = nd[q].z;
         }
     }
     if constexpr (PASS == kPassAll) {
@@ -583,7 +648,7 @@ __device__ __forceinline__ bool dims_fit_queue(const int (&dim)[3])
 // pointers, (C+1)%3, (C+2)%3 and C, into the record arrays (vertex or face i is 3 rows = 96
 // scalars further on; the normals follow the vertices at 12 rows = 384 scalars), so a fetch is
 // three loads at fixed offsets and no selects.  T = float reads the float32 record; T = double
-// the guarded pass's exact vertices.
+// the guarded pass's exact vertices (no normals: the float64 clip needs none).
 template <class T>
 struct RecordRun {
     const T *va, *vb, *vc;  // row pointers
@@ -598,15 +663,14 @@ struct RecordRun {
     }
 };
 static_assert(offsetof(WarpSmem, n) == offsetof(WarpSmem, v) + 384 * sizeof(float), "RecordRun reads n after v");
-static_assert(offsetof(GuardSmem, n) == offsetof(GuardSmem, v) + 384 * sizeof(double), "RecordRun reads n after v");
 
 template <class T>
-__device__ __forceinline__ RecordRun<T> record_run(WarpSmem *S, int t, int C, float la, float lb, float lc)
+__device__ __forceinline__ RecordRun<T> record_run(WarpSmem *S, int t, int C, T la, T lb, T lc)
 {
     const T *rows;
     if constexpr (sizeof(T) == sizeof(float)) rows = &S->v[0][t];
     else rows = &guard_smem(S)->v[0][t];
-    return RecordRun<T>{rows + 32 * axis_a(C), rows + 32 * axis_b(C), rows + 32 * C, (T)la, (T)lb, (T)lc};
+    return RecordRun<T>{rows + 32 * axis_a(C), rows + 32 * axis_b(C), rows + 32 * C, la, lb, lc};
 }
 
 // Lane `lane`'s edge slots of the column clip.
@@ -754,6 +818,22 @@ __device__ __forceinline__ void clip_round(const DepositParams &P, WarpSmem *S, 
     __syncwarp();
 }
 
+// The face terms of a pass's clips, and a float32 value as its scalar.
+template <class T>
+struct FaceOf {
+    using type = FaceRun<kRun, float>;
+};
+template <>
+struct FaceOf<double> {
+    using type = FaceRun64<kRun>;
+};
+template <class T>
+__device__ __forceinline__ T widen(float x)
+{
+    if constexpr (sizeof(T) == sizeof(float)) return x;
+    else return f64_widen(x);
+}
+
 // The run word (ra.w): record t (bits 0-4), faces to clip (bits 5-8), cells kw (9-10), axis C
 // (11-12), lo_open (13).
 constexpr int kRunMask = 5, kRunLen = 9, kRunAxis = 11, kRunOpen = 13;
@@ -791,8 +871,8 @@ __device__ __forceinline__ void job_round(const DepositParams &P, WarpSmem *S, i
     const unsigned starts = __reduce_or_sync(kFull, fits ? 1u << first : 0u);
 
     // ---- one face per lane
-    FaceRun<kRun, T> fr;
-    face_none<kRun, T>(fr);
+    typename FaceOf<T>::type fr;
+    face_none(fr);
     T qz = T(0);
     {
         const int r = __popc(starts & le_mask) - 1;
@@ -806,24 +886,32 @@ __device__ __forceinline__ void job_round(const DepositParams &P, WarpSmem *S, i
             const int slot = (head + r) & 63;
             const float4 ra = S->ra[slot], rb = S->rb[slot];
             const int t = (int)(w & 31u), C = (int)((w >> kRunAxis) & 3u);
-            const RecordRun<T> src = record_run<T>(S, t, C, ra.x, ra.y, ra.z);
             RunFrame<T> F;
-            F.qx = (T)rb.x;
-            F.qy = (T)rb.y;
-            F.qz = (T)rb.z;
-            if constexpr (sizeof(T) == sizeof(float)) F.l0 = rb.w;
-            else F.l0 = guard_smem(S)->l0[slot];
-            F.lx = (T)S->lx[t];
-            F.ly = (T)S->ly[t];
+            F.qx = widen<T>(rb.x);
+            F.qy = widen<T>(rb.y);
+            F.qz = widen<T>(rb.z);
+            F.l0 = widen<T>(rb.w);
+            F.lx = widen<T>(S->lx[t]);
+            F.ly = widen<T>(S->ly[t]);
             F.K = (int)((w >> kRunLen) & 3u);
             F.j0 = ((w >> kRunOpen) & 1u) ? 0 : 1;
             qz = F.qz;
             int ia, ib, ic;
             face_vertices(f, ia, ib, ic);
-            const P3<T> q = mk<T>(F.qx, F.qy, F.qz);
-            const P3<T> a = sub(src.vtx(ia), q), b = sub(src.vtx(ib), q), c = sub(src.vtx(ic), q);
-            const P3<T> nf = src.nrm(f);
-            if (face_meets_column<T>(a, b, c, nf.z, F)) face_run<kRun, T>(a, b, c, nf, F, lane_slots(S, lane, T(0)), fr);
+            if constexpr (sizeof(T) == sizeof(float)) {
+                const RecordRun<float> src = record_run<float>(S, t, C, ra.x, ra.y, ra.z);
+                const P3<float> q = mk<float>(F.qx, F.qy, F.qz);
+                const P3<float> a = sub(src.vtx(ia), q), b = sub(src.vtx(ib), q), c = sub(src.vtx(ic), q);
+                const P3<float> nf = src.nrm(f);
+                if (face_meets_column<float>(a, b, c, nf.z, F))
+                    face_run<kRun, float>(a, b, c, nf, F, lane_slots(S, lane, 0.f), fr);
+            } else {
+                // straight into the frame: first cell + q is exact
+                const RecordRun<double> src = record_run<double>(S, t, C, widen<double>(ra.x) + F.qx,
+                                                                 widen<double>(ra.y) + F.qy, widen<double>(ra.z) + F.qz);
+                face_run_f64<kRun>(src.vtx(ia), src.vtx(ib), src.vtx(ic), F, guard_smem(S)->tol[t],
+                                   lane_slots(S, lane, 0.0), fr);
+            }
         }
     }
     __syncwarp();
@@ -851,14 +939,18 @@ __device__ __forceinline__ void job_round(const DepositParams &P, WarpSmem *S, i
             from = e & 31;
             j = (e >> 5) + lane - p;
         }
-        const T nx = __shfl_sync(kFull, fr.nx, from), ny = __shfl_sync(kFull, fr.ny, from),
-                nz = __shfl_sync(kFull, fr.nz, from), ef = __shfl_sync(kFull, fr.ef, from),
-                fq = __shfl_sync(kFull, qz, from);
+        const T fq = __shfl_sync(kFull, qz, from);
         const int ne = __shfl_sync(kFull, fr.n, from);
         T g = T(0);
-        if (lane < nfan) {
-            const T cj = (T)j - fq;
-            g = level_fan<OCT, T>(lane_slots(S, from, T(0)), ne, cj, fan_anchor<T>(nx, ny, nz, ef, cj), nx, ny);
+        if constexpr (sizeof(T) == sizeof(float)) {
+            const float nx = __shfl_sync(kFull, fr.nx, from), ny = __shfl_sync(kFull, fr.ny, from),
+                        nz = __shfl_sync(kFull, fr.nz, from), ef = __shfl_sync(kFull, fr.ef, from);
+            if (lane < nfan) {
+                const float cj = (float)j - fq;
+                g = level_fan<OCT, float>(lane_slots(S, from, 0.f), ne, cj, fan_anchor<float>(nx, ny, nz, ef, cj), nx, ny);
+            }
+        } else {
+            if (lane < nfan) g = level_fan_f64(lane_slots(S, from, 0.0), ne, widen<double>((float)j) - fq);
         }
 #pragma unroll
         for (int i = 0; i <= kRun; ++i) {
@@ -876,8 +968,13 @@ __device__ __forceinline__ void job_round(const DepositParams &P, WarpSmem *S, i
     if (lane < J) {
 #pragma unroll
         for (int i = 0; i <= kRun; ++i) comb[i][lane] = fr.k6[i];
-        comb[3][lane] = fr.zmin;
-        comb[4][lane] = fr.zmax;
+        if constexpr (sizeof(T) == sizeof(float)) {
+            comb[3][lane] = fr.zmin;
+            comb[4][lane] = fr.zmax;
+        } else {
+            comb[3][lane] = __longlong_as_double(fr.kmin);
+            comb[4][lane] = __longlong_as_double(fr.kmax);
+        }
         comb[5][lane] = fr.m6;
     }
     __syncwarp();
@@ -889,21 +986,32 @@ __device__ __forceinline__ void job_round(const DepositParams &P, WarpSmem *S, i
         const int kw = (int)((w >> kRunLen) & 3u);
         if (r < R && j < kw) {
             const int nf = __popc((w >> kRunMask) & 15u);
-            T s0 = T(0), s1 = T(0), colmin = T(1e30), colmax = T(-1e30), msum = T(0);
+            T s0 = T(0), s1 = T(0), msum = T(0);
+            float colmin = 1e30f, colmax = -1e30f;
+            long long kmin = kKeyMax, kmax = kKeyMin;
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 if (i < nf) {
                     s0 += comb[j][j0 + i];
                     s1 += comb[j + 1][j0 + i];
-                    colmin = fmin(colmin, comb[3][j0 + i]);
-                    colmax = fmax(colmax, comb[4][j0 + i]);
                     msum += comb[5][j0 + i];
+                    if constexpr (sizeof(T) == sizeof(float)) {
+                        colmin = fminf(colmin, comb[3][j0 + i]);
+                        colmax = fmaxf(colmax, comb[4][j0 + i]);
+                    } else {
+                        const long long kl = __double_as_longlong(comb[3][j0 + i]), kh = __double_as_longlong(comb[4][j0 + i]);
+                        kmin = kl < kmin ? kl : kmin;
+                        kmax = kh > kmax ? kh : kmax;
+                    }
                 }
             }
             const int slot = (head + r) & 63;
             const float4 ra = S->ra[slot];
-            const T fq = (T)S->rb[slot].z;
-            const T vol = level_volume<T>((T)j - fq, (T)(j + 1) - fq, s0, s1, colmin, colmax, msum);
+            const float fq = S->rb[slot].z;
+            const float c0 = (float)j - fq, c1 = (float)(j + 1) - fq;  // exact: multiples of 1/256
+            T vol;
+            if constexpr (sizeof(T) == sizeof(float)) vol = level_volume<float>(c0, c1, s0, s1, colmin, colmax, msum);
+            else vol = level_volume_f64(widen<double>(c0), widen<double>(c1), s0, s1, kmin, kmax, msum);
             const int t = (int)(w & 31u), C = (int)((w >> kRunAxis) & 3u);
             const int la = (int)ra.x, lb = (int)ra.y, lc = (int)ra.z + j;
             const int ex = C == 0 ? lc : (C == 1 ? lb : la), ey = C == 1 ? lc : (C == 2 ? lb : la),
@@ -1029,7 +1137,6 @@ __device__ __forceinline__ void coop_runs(const DepositParams &P, WarpSmem *S, i
         const int idx = b0 + lane;
         unsigned word = 0;
         float4 ra = make_float4(0.f, 0.f, 0.f, 0.f), rb = ra;
-        double l0 = 0.0;
         if (idx < total) {
             const int t = pair_record(S, idx);
             int local = idx - S->start[t] + skip;
@@ -1058,16 +1165,20 @@ __device__ __forceinline__ void coop_runs(const DepositParams &P, WarpSmem *S, i
                 P3<float> p[4];
                 unsigned up = 0, flat = 0;
 #pragma unroll
+                for (int q = 0; q < 4; ++q) p[q] = near.vtx(q);
+#pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    p[q] = near.vtx(q);
+                    float nz;
                     if constexpr (sizeof(T) == sizeof(float)) {
-                        const float nz = near.vc[384 + 96 * q];
-                        up |= nz > 0.f ? 1u << q : 0u;
+                        nz = near.vc[384 + 96 * q];
                         flat |= nz == 0.f ? 1u << q : 0u;  // vertical: no projected area
                     } else {
-                        const double *nz = &guard_smem(S)->n[3 * q + C][t];
-                        up |= __double2hiint(*nz) >= 0 ? 1u << q : 0u;
+                        // (the guarded pass may have turned the vertices over)
+                        int ia, ib, ic;
+                        face_vertices(q, ia, ib, ic);
+                        nz = (p[ib].x - p[ia].x) * (p[ic].y - p[ia].y) - (p[ib].y - p[ia].y) * (p[ic].x - p[ia].x);
                     }
+                    up |= nz > 0.f ? 1u << q : 0u;
                 }
                 unsigned mask = face_mask(p, up) & ~flat;
                 if (STATS && mask == 0u) mask = 1u;  // counted as a run all the same
@@ -1076,10 +1187,10 @@ __device__ __forceinline__ void coop_runs(const DepositParams &P, WarpSmem *S, i
                     word = (unsigned)t | (mask << kRunMask) | ((unsigned)kw << kRunLen) | ((unsigned)C << kRunAxis) |
                            (lo_open ? 1u << kRunOpen : 0u);
                     ra = make_float4((float)la, (float)lb, (float)lc, __uint_as_float(word));
-                    const RecordRun<T> src = record_run<T>(S, t, C, ra.x, ra.y, ra.z);
-                    const RunFrame<T> F = run_frame<T>(src, (T)S->lx[t], (T)S->ly[t], kw, lo_open);
-                    rb = make_float4((float)F.qx, (float)F.qy, (float)F.qz, (float)F.l0);
-                    l0 = (double)F.l0;
+                    // (the float64 clip takes the float32 frame too: any nearby origin and
+                    // reference plane serve)
+                    const RunFrame<float> F = run_frame<float>(near, S->lx[t], S->ly[t], kw, lo_open);
+                    rb = make_float4(F.qx, F.qy, F.qz, F.l0);
                 }
             }
         }
@@ -1088,7 +1199,6 @@ __device__ __forceinline__ void coop_runs(const DepositParams &P, WarpSmem *S, i
             const int slot = (head + qn + __popc(bal & lt_mask)) & 63;
             S->ra[slot] = ra;
             S->rb[slot] = rb;
-            if constexpr (sizeof(T) != sizeof(float)) guard_smem(S)->l0[slot] = l0;
         }
         qn += __popc(bal);
         jobs += (int)__reduce_add_sync(kFull, (unsigned)__popc((word >> kRunMask) & 15u));
@@ -1175,7 +1285,7 @@ __device__ __forceinline__ void coop_cells(const DepositParams &P, WarpSmem *S, 
 
 // Each warp's shared memory is a WarpSmem; in the guarded pass a GuardSmem takes the place of
 // its float slots (the struct's last member, which that pass never touches) and runs past the
-// struct's end: 26 KB a warp, two 4-warp blocks an SM.
+// struct's end: 23 KB a warp, two 4-warp blocks an SM.
 constexpr size_t kGuardWarpBytes = offsetof(WarpSmem, poly) + sizeof(GuardSmem);
 static_assert(offsetof(WarpSmem, poly) % 16 == 0 && kGuardWarpBytes % 16 == 0 && sizeof(WarpSmem) % 16 == 0,
               "warp blocks of shared memory must keep 16-byte alignment");

@@ -81,7 +81,6 @@ __global__ void __launch_bounds__(kCoopThreads, MINB) k_warp_coop(const DepositP
     Counters cnt;
     if (STATS) cnt.zero();
     cnt.zero_mass();
-    const int nsub = (P.src == SRC_TETS) ? 1 : 6;
     // binned schedule: items [0, n_chunks) are pieces of split tetrahedra (largest work
     // first), the rest are the rows; tetrahedra the bin pass queued are skipped there
     int64_t n_chunks = 0, q = 0;
@@ -95,7 +94,8 @@ __global__ void __launch_bounds__(kCoopThreads, MINB) k_warp_coop(const DepositP
     // when it listed all of them
     const int64_t listed = (!FIRST && !BINNED) ? listed_guarded(P) : -1;
     const bool LIST = listed >= 0;
-    const int64_t n_items = LIST ? (listed + 31) / 32 : P.n_items;
+    const int per = LIST ? listed_per_item(listed) : P.group;  // tetrahedra per item
+    const int64_t n_items = LIST ? (listed + per - 1) / per : P.n_items;
 
     for (;;) {
         unsigned long long item = 0;
@@ -107,58 +107,41 @@ __global__ void __launch_bounds__(kCoopThreads, MINB) k_warp_coop(const DepositP
             if ((int64_t)item >= n_items) break;
         }
 
-        // the 32 units (cubes or tetrahedra) of this item
+        // this item's tetrahedra, one per lane: of `group` cubes one Kuhn tetrahedron s each, of
+        // a tetrahedron source `group` tetrahedra, of the list `per` listed ones
         int64_t unit = -1;
         int64_t ci = 0, cj = 0, ck = 0;
-        int s_listed = 0;
+        int s = 0;
         if (is_chunk) {
             // nothing: chunk_setup below
         } else if (LIST) {
-            // one listed tetrahedron per lane: its id decodes like the ids below
-            const int64_t k = (int64_t)item * 32 + lane;
-            if (k < listed) {
-                const int64_t id = P.guard_list[k];
-                if (P.src == SRC_TETS) {
-                    unit = id;
-                } else {
-                    const int64_t u = id / 6;
-                    s_listed = (int)(id % 6);
-                    if (P.src == SRC_LATTICE) {
-                        ci = u % P.nc[0];
-                        cj = (u / P.nc[0]) % P.nc[1];
-                        ck = u / (P.nc[0] * P.nc[1]);
-                        unit = 1;
-                    } else if (cube_of_unit(P, u, ci, cj, ck)) {
-                        unit = u;
-                    }
+            // its id decodes like the ids below
+            const int64_t k = (int64_t)item * per + lane;
+            if (lane < per && k < listed) {
+                unit = P.guard_list[k];
+                if (P.src != SRC_TETS) {
+                    s = (int)(unit % 6);
+                    unit /= 6;
+                    if (!cube_of_unit(P, unit, ci, cj, ck)) unit = -1;
                 }
             }
-        } else if (P.src == SRC_LATTICE) {
-            // rows of 32 cubes along x
-            const int64_t segs = (P.nc[0] + 31) / 32;
-            const int64_t row = (int64_t)item / segs, seg = (int64_t)item % segs;
-            const int64_t i = seg * 32 + lane;
-            if (i < P.nc[0]) {
-                ci = i;
-                cj = row % P.nc[1];
-                ck = row / P.nc[1];
-                unit = 1;
-            }
         } else {
-            const int64_t u = (int64_t)item * 32 + lane;
-            if (u < P.n_units) {
+            int64_t g = (int64_t)item;
+            if (P.src != SRC_TETS) {  // the 6 tetrahedra of a group of cubes are neighbouring items
+                s = (int)(item % 6);
+                g = (int64_t)(item / 6);
+            }
+            const int64_t u = g * per + lane;
+            if (lane < per && u < P.n_units) {
                 unit = u;
-                if (P.src == SRC_CUBE_LIST && !cube_of_unit(P, u, ci, cj, ck)) {
+                if (P.src != SRC_TETS && !cube_of_unit(P, u, ci, cj, ck)) {
                     set_error(P.ws, 3, (int)(u & 0x7fffffff));
                     unit = -1;
                 }
             }
         }
 
-        const int nsub_item = (is_chunk || LIST) ? 1 : nsub;
-#pragma unroll 1
-        for (int si = 0; si < nsub_item; ++si) {
-            const int s = LIST ? s_listed : si;
+        {
             // ---- 1. one tetrahedron per lane (or the queued tetrahedron's chunk on lane 0)
             int npairs = 0, skip = 0;
             double m_t = 0.0;
@@ -171,8 +154,7 @@ __global__ void __launch_bounds__(kCoopThreads, MINB) k_warp_coop(const DepositP
                 P3<float> v[4];
                 int base[3];
                 // tetrahedron id as the bin pass numbers it (and the guarded-tetrahedron list)
-                tid = (P.src == SRC_TETS) ? unit
-                                          : 6 * ((P.src == SRC_LATTICE) ? ci + P.nc[0] * (cj + P.nc[1] * ck) : unit) + s;
+                tid = (P.src == SRC_TETS) ? unit : 6 * unit + s;
                 if (P.src == SRC_TETS) {
                     explicit_tet<float>(P, unit, v, base);
                     m_t = P.tet_mass[unit];

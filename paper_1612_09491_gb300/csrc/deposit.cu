@@ -324,8 +324,8 @@ __global__ void k_finish(double *__restrict__ out, long long n, const Workspace 
 {
     double f = 1.0;
     if (SCALE) {
-        const double dep = ws->mass_deposited;
-        if (dep > 0.0) f = ws->mass_target / dep;
+        const double dep = ws->mass_deposited + ws->mass_deposited_lo;
+        if (dep > 0.0) f = (ws->mass_target + ws->mass_target_lo) / dep;
         else if (!COMP) return;
     }
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {

@@ -34,6 +34,7 @@ struct Workspace {
     double mass_dropped;
     double mass_target;     // sum of m_t over processed tetrahedra (FP32 mass renormalisation)
     double mass_deposited;  // sum of every computed deposit, in the grid or dropped
+    double mass_target_lo, mass_deposited_lo;  // the rounding errors of the additions to the two sums
     int error_code;                    // first device-side error (0 = none)
     int error_detail;
     // binned schedule
@@ -81,6 +82,8 @@ struct DepositParams {
     int64_t fine;              // F = 2^max_level
     // scheduling
     int64_t n_items;
+    int32_t group;             // cubes (tetrahedra of SRC_TETS) that one work item of the warp kernels takes
+    int32_t subs;              // octree: Kuhn tetrahedra of each cube that an item takes (1 or 6); else 1
     Workspace *ws;
     // binned schedule: tetrahedra whose bounding box has more than split_cells cells are
     // queued by the bin pass and split into work items of chunk_cells cells
