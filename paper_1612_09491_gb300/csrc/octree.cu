@@ -662,15 +662,45 @@ __global__ void __launch_bounds__(128, MINB) k_oct_warp(const DepositParams P)
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ int64_t hist_offset(int level) { return (int64_t)64 * ((((int64_t)1) << (3 * level)) - 1) / 7; }
 
+// The finest decision-level node of a tetrahedron's vertex centroid in float64, for centroids
+// within float32 rounding of a node boundary.
+__device__ __noinline__ int3 exact_node(const DepositParams &P, int64_t ci, int64_t cj, int64_t ck, int s, int top)
+{
+    float x[4][3];
+    lattice_positions(P, ci, cj, ck, s, x);
+    const double inv_box = 1.0 / P.box, scale = (double)((int64_t)1 << top);
+    int c[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        double d[4];
+#pragma unroll
+        for (int q = 1; q < 4; ++q) {
+            const int sh = P.periodic ? image_shift(P, x[q][a], x[0][a]) : 0;
+            d[q] = ((double)x[q][a] - (double)x[0][a]) + (double)sh * P.box;
+        }
+        double cen = (double)x[0][a] + 0.25 * ((d[1] + d[2]) + d[3]);
+        cen -= P.box * floor(cen * inv_box);
+        if (!(cen < P.box) || !(cen >= 0.0)) cen = 0.0;
+        const int64_t n = (int64_t)floor(cen * scale * inv_box), nn = (int64_t)1 << top;
+        c[a] = (int)(n < 0 ? 0 : (n >= nn ? nn - 1 : n));
+    }
+    return make_int3(c[0], c[1], c[2]);
+}
+
 // One pass over the tetrahedra: per level 0 .. max_level-1, the node that holds the
 // tetrahedron's vertex centroid and the 64-bin log10 histogram bin of its mean edge length
 // in that level's cells.  A lane takes one Lagrangian cube (a warp: 32 neighbouring cubes of a
 // row) and its 6 Kuhn tetrahedra, which all start at corner 000: the 7 other corners are
-// loaded once, unwrapped once (offsets from corner 000 formed in float64 and rounded to
-// float32; a bin is 24% wide), and the 19 distinct edges serve all 6 tetrahedra.  The
-// centroid is summed in float64 from the same offsets, and the nodes of the coarser levels
-// are the finest level's node coordinates shifted (scaling by 2^l commutes with rounding).
-// Equal (node, bin) keys are merged in the warp before one atomic per key.
+// loaded once and unwrapped once, and the 19 distinct edges serve all 6 tetrahedra.  The nodes
+// of the coarser levels are the finest level's node coordinates shifted.  Equal (node, bin)
+// keys are merged in the warp before one atomic per key.
+//
+// The float64 centroids bound this kernel (16 cycles a warp instruction: 11.2 ms for 256^3,
+// the float64 pipe 83% busy), so nodes and bins come from float32 and only what lies within
+// the rounding of a boundary is decided by the float64 centroid and the level's own log10.
+// Float32 errors: below 4e-7 of the box and of the position for a centroid, below 2e-5 of a bin
+// for the shifted logarithm; the margins are 2e-6 and 4e-5.  Measured: the 256^3 octree build and
+// deposit 277 -> 270.5 ms.
 __global__ void __launch_bounds__(256) k_tet_size_hist(const DepositParams P, unsigned *__restrict__ hist)
 {
     __shared__ unsigned sh[64 + 512];  // levels 0 and 1 aggregated per block
@@ -678,55 +708,40 @@ __global__ void __launch_bounds__(256) k_tet_size_hist(const DepositParams P, un
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const int levels = P.max_level;  // decisions are made for levels 0 .. max_level-1
-    const double inv_box = 1.0 / P.box;
     const float h0 = (float)(P.box / (double)P.bc);
-    const bool rows = P.src == SRC_LATTICE;
-    const int64_t segs = (P.nc[0] + 31) / 32;
-    const int64_t n_items = rows ? segs * P.nc[1] * P.nc[2] : (P.n_units + 31) / 32;
+    const int64_t n_items = (P.n_units + 31) / 32;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     const int top = levels > 0 ? levels - 1 : 0;  // the finest decision level
-    const double top_scale = (double)((int64_t)1 << top);
+    const float nodes = (float)(1 << top), to_node = (float)((double)(1 << top) / P.box);
+    const float near = 0.49f * (float)P.box;
     // whole warps iterate together (the merge below needs every lane)
     for (int64_t item = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); item < n_items; item += warps) {
         int64_t ci = 0, cj = 0, ck = 0;
-        bool ok = false;
-        if (rows) {
-            const int64_t row = item / segs, i = (item % segs) * 32 + lane;
-            if (i < P.nc[0]) {
-                ci = i;
-                cj = row % P.nc[1];
-                ck = row / P.nc[1];
-                ok = true;
-            }
-        } else {
-            const int64_t u = item * 32 + lane;
-            ok = u < P.n_units && cube_of_unit(P, u, ci, cj, ck);
-        }
+        const int64_t u = item * 32 + lane;
+        const bool ok = u < P.n_units && cube_of_unit(P, u, ci, cj, ck);
         // corner c = (bit 0: +x, bit 1: +y, bit 2: +z): offsets from corner 000
         float x0[3] = {0.f, 0.f, 0.f}, r[8][3];
-        double d[8][3];
 #pragma unroll
-        for (int a = 0; a < 3; ++a) { r[0][a] = 0.f; d[0][a] = 0.0; }
+        for (int a = 0; a < 3; ++a) r[0][a] = 0.f;
         if (ok) {
+            const int64_t r1 = 3 * P.n[0], r2 = r1 * P.n[1];
+            const int64_t d0 = (P.periodic && ci + 1 == P.n[0]) ? 3 - r1 : 3;
+            const int64_t d1 = (P.periodic && cj + 1 == P.n[1]) ? r1 - r2 : r1;
+            const int64_t d2 = (P.periodic && !P.slab && ck + 1 == P.n[2]) ? r2 - r2 * P.n[2] : r2;
+            const float *p0 = P.pos + (3 * ci + r1 * cj + r2 * ck);
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
-                int64_t i = ci + (c & 1), j = cj + ((c >> 1) & 1), kk = ck + ((c >> 2) & 1);
-                if (P.periodic) {
-                    i = wrap_idx(i, P.n[0]);
-                    j = wrap_idx(j, P.n[1]);
-                    if (!P.slab) kk = wrap_idx(kk, P.n[2]);
-                }
-                const float *pp = P.pos + 3 * (i + P.n[0] * (j + P.n[1] * kk));
-                float x[3] = {__ldg(pp), __ldg(pp + 1), __ldg(pp + 2)};
+                const float *pp = p0 + ((c & 1) ? d0 : 0) + ((c & 2) ? d1 : 0) + ((c & 4) ? d2 : 0);
 #pragma unroll
                 for (int a = 0; a < 3; ++a) {
+                    const float x = __ldg(pp + a);
                     if (c == 0) {
-                        x0[a] = x[a];
+                        x0[a] = x;
                     } else {
-                        const double raw = (double)x[a] - (double)x0[a];
-                        const int sh = P.periodic ? ((raw >= 0.5 * P.box) ? -1 : ((raw < -0.5 * P.box) ? 1 : 0)) : 0;
-                        d[c][a] = raw + (double)sh * P.box;
-                        r[c][a] = (float)d[c][a];
+                        float d = x - x0[a];
+                        if (P.periodic && !(fabsf(d) < near))
+                            d = (float)(((double)x - (double)x0[a]) + (double)image_shift(P, x, x0[a]) * P.box);
+                        r[c][a] = d;
                     }
                 }
             }
@@ -737,8 +752,8 @@ __global__ void __launch_bounds__(256) k_tet_size_hist(const DepositParams P, un
             kuhn_offsets(s, o1, o2);
             const int c1 = o1[0] | (o1[1] << 1) | (o1[2] << 2), c2 = o2[0] | (o2[1] << 1) | (o2[2] << 2);
             const int cq[4] = {0, c1, c2, 7};
-            float me = 0.f;  // mean edge length in level-0 cells
-            int64_t top_c[3] = {0, 0, 0};
+            float me = 0.f, y0 = 0.f;  // mean edge length in level-0 cells, and its place among the bins
+            int3 at = make_int3(0, 0, 0);
             if (ok) {
                 float es = 0.f;
 #pragma unroll
@@ -750,34 +765,40 @@ __global__ void __launch_bounds__(256) k_tet_size_hist(const DepositParams P, un
                         es += sqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
                     }
                 me = es * (1.f / 6.f) / h0;
+                y0 = (log10f(me) + 3.0f) * (64.0f / 6.0f);
+                bool sure = true;
+                int c[3];
 #pragma unroll
                 for (int a = 0; a < 3; ++a) {
-                    double cen = (double)x0[a] + 0.25 * ((d[c1][a] + d[c2][a]) + d[7][a]);
-                    cen -= P.box * floor(cen * inv_box);
-                    if (!(cen < P.box) || !(cen >= 0.0)) cen = 0.0;
-                    int64_t c = (int64_t)floor(cen * top_scale * inv_box);
-                    const int64_t nn = (int64_t)1 << top;
-                    top_c[a] = c < 0 ? 0 : (c >= nn ? nn - 1 : c);
+                    const float v = (x0[a] + 0.25f * ((r[c1][a] + r[c2][a]) + r[7][a])) * to_node;
+                    const float fl = floorf(v), part = v - fl, margin = 2e-6f * (nodes + fabsf(v));
+                    sure = sure && part > margin && part < 1.f - margin;  // (false for NaN)
+                    c[a] = (int)fl & ((1 << top) - 1);
                 }
+                at = make_int3(c[0], c[1], c[2]);
+                if (!sure) at = exact_node(P, ci, cj, ck, s, top);
             }
             for (int l = 0; l < levels; ++l) {
                 unsigned long long key = ~0ull - (unsigned long long)lane;  // lanes without a cube match nothing
+                unsigned node = 0;
                 int bin = 0;
-                int64_t node = 0;
                 if (ok) {
-                    const int sh = top - l;
-                    node = (top_c[0] >> sh) + ((top_c[1] >> sh) << l) + ((top_c[2] >> sh) << (2 * l));
-                    // a level-l cell is 2^-l of a level-0 cell (an exact float scaling)
-                    bin = (int)floorf((log10f(ldexpf(me, l)) + 3.0f) * (64.0f / 6.0f));
+                    const int down = top - l;
+                    node = (unsigned)(at.x >> down) + ((unsigned)(at.y >> down) << l) + ((unsigned)(at.z >> down) << (2 * l));
+                    // a level-l cell is 2^-l of a level-0 cell: 64/6 log10(2) bins a level
+                    float y = fmaf((float)l, 3.2109866f, y0);
+                    const float part = y - floorf(y);
+                    if (!(part > 4e-5f && part < 1.f - 4e-5f) && l > 0) y = (log10f(ldexpf(me, l)) + 3.0f) * (64.0f / 6.0f);
+                    bin = (int)floorf(y);
                     bin = bin < 0 ? 0 : (bin > 63 ? 63 : bin);
                     key = (unsigned long long)node * 64 + (unsigned long long)bin;
                 }
                 const unsigned peers = __match_any_sync(kFull, key);
-                if (ok && lane == __ffs(peers) - 1) {
+                if (ok && lane == __ffs((int)peers) - 1) {
                     const unsigned cnt = (unsigned)__popc(peers);
                     if (l == 0) atomicAdd(&sh[bin], cnt);
                     else if (l == 1) atomicAdd(&sh[64 + node * 64 + bin], cnt);
-                    else atomicAdd(&hist[hist_offset(l) + node * 64 + bin], cnt);
+                    else atomicAdd(&hist[hist_offset(l) + (int64_t)node * 64 + bin], cnt);
                 }
             }
         }
