@@ -166,6 +166,11 @@ void fill_grid(pse::DepositParams &p, const int64_t grid_n[3], double box)
 // segment of 32 cubes with all six tetrahedra: 16^3 on 32^3 0.86 -> 0.46 ms, 32^3 on 64^3 0.92 ->
 // 0.56 ms, 48^3 on 384^3, whose rows fill three quarters of a warp, 31.0 -> 18.3 ms, 256^3 on
 // 128^3 64.7 -> 56.4 ms.)
+// The FP32 pass on a uniform grid paces its blocks (coop.cuh) up to this many cells a cube.  160^3
+// cubes, unpaced and paced: 0.5 cells 18.4 and 16.7 ms, 1 cell 21.7 and 20.5, 2 cells 27.5 and
+// 27.4, 4 cells 38.8 and 39.7.
+constexpr double kPaceCells = 2.0;
+
 void set_items(pse::DepositParams &p)
 {
     constexpr int64_t kWarps = 152 * 16;
@@ -175,6 +180,11 @@ void set_items(pse::DepositParams &p)
     const int64_t groups = (p.n_units + p.group - 1) / p.group;
     p.subs = (p.leaves && groups >= 4 * kWarps) ? 6 : 1;
     p.n_items = groups * (nsub / (p.leaves ? p.subs : 1));
+    if (p.slab) return;  // a slab keeps the whole lattice's choice
+    p.pace = (!p.leaves && p.src != pse::SRC_TETS &&
+              (double)p.g[0] * (double)p.g[1] * (double)p.g[2] <= kPaceCells * (double)p.nc[0] * (double)p.nc[1] *
+                                                                      (double)p.nc[2])
+                 ? 1 : 0;
 }
 
 // ---------------------------------------------------------------------------

@@ -103,6 +103,32 @@ __device__ __forceinline__ int image_shift(const DepositParams &P, float v, floa
     return (d >= 0.5 * P.box) ? -1 : ((d < -0.5 * P.box) ? 1 : 0);
 }
 
+// The nine shifts of vertices 1..3 against vertex 0, 2 bits each (0, 1: +box, 2: -box; see
+// shift_of), for the tetrahedra that may_shift picks out; out of line to keep hot code small.
+__device__ __noinline__ unsigned far_shifts(double box, float a0, float a1, float a2, float b0, float b1, float b2,
+                                            float c0, float c1, float c2, float d0, float d1, float d2)
+{
+    const float v0[3] = {a0, a1, a2}, v[9] = {b0, b1, b2, c0, c1, c2, d0, d1, d2};
+    unsigned bits = 0;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        const double d = (double)v[i] - (double)v0[i % 3];
+        bits |= ((d >= 0.5 * box) ? 2u : ((d < -0.5 * box) ? 1u : 0u)) << (2 * i);
+    }
+    return bits;
+}
+__device__ __forceinline__ unsigned tet_shift_bits(const DepositParams &P, const float (&x)[4][3])
+{
+    if (!may_shift(P, x)) return 0u;
+    return far_shifts(P.box, x[0][0], x[0][1], x[0][2], x[1][0], x[1][1], x[1][2], x[2][0], x[2][1], x[2][2], x[3][0],
+                      x[3][1], x[3][2]);
+}
+__device__ __forceinline__ int shift_of(unsigned bits, int q, int a)
+{
+    const int b = q == 0 ? 0 : (int)((bits >> (2 * (3 * (q - 1) + a))) & 3u);
+    return b == 2 ? -1 : b;
+}
+
 // Vertices of tetrahedron s of Lagrangian cube (ci, cj, ck), in grid units relative to
 // the base cell (the cell holding corner 000), each corner at its periodic image nearest to
 // corner 000.
@@ -129,14 +155,12 @@ __device__ __forceinline__ void lattice_tet(const DepositParams &P, int64_t ci, 
     for (int q = 0; q < 4; ++q)
 #pragma unroll
         for (int a = 0; a < 3; ++a) place(q, a, -base[a]);
-    if (may_shift(P, x)) {
+    const unsigned shifts = tet_shift_bits(P, x);
+    if (shifts != 0) {
 #pragma unroll
         for (int q = 1; q < 4; ++q)
 #pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                const int shift = image_shift(P, x[q][a], x[0][a]);
-                if (shift != 0) place(q, a, shift * (int)P.g[a] - base[a]);
-            }
+            for (int a = 0; a < 3; ++a) place(q, a, shift_of(shifts, q, a) * (int)P.g[a] - base[a]);
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {

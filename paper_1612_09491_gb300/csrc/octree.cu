@@ -321,53 +321,52 @@ constexpr unsigned kWalkDone = 0xffffu;  // at[2] >> 16 once every node has been
 __device__ __forceinline__ bool walk_done(const LeafWalk &w) { return (w.at[2] >> 16) == kWalkDone; }
 __device__ __forceinline__ void walk_end(LeafWalk &w) { w.at[2] = kWalkDone << 16; }
 
-__device__ __forceinline__ int walk_shift(unsigned shifts, int q, int a)
+// The finest nodes that coordinates x0..x3 (axis a) of a tetrahedron cover, in float64: for
+// periodic shifts and for coordinates within float32 rounding of a node boundary; out of line.
+// x: LeafWalk::first, y: LeafWalk::at, or -1 in y if a coordinate is not finite (or 2^21 boxes and
+// more away, where float32 holds no position).
+__device__ __noinline__ int2 exact_nodes(const DepositParams &P, unsigned shifts, int a, float x0, float x1, float x2,
+                                         float x3)
 {
-    if (q == 0) return 0;
-    const int b = (shifts >> (2 * (3 * (q - 1) + a))) & 3;
-    return b == 2 ? -1 : b;
+    const double u1 = (double)x1 + (double)shift_of(shifts, 1, a) * P.box, u2 = (double)x2 + (double)shift_of(shifts, 2, a) * P.box,
+                 u3 = (double)x3 + (double)shift_of(shifts, 3, a) * P.box, u0 = (double)x0;
+    const double fine = (double)P.fine, scale = fine / P.box;
+    const double f0 = floor(fmin(fmin(u0, u1), fmin(u2, u3)) * scale), f1 = floor(fmax(fmax(u0, u1), fmax(u2, u3)) * scale);
+    const double image = floor(f0 / fine);  // exact: the number of finest nodes is a power of two
+    const double span = f1 - f0;
+    if (!(fabs(image) < 2097152.0 && span < 65535.0)) return make_int2(0, -1);
+    return make_int2((int)(f0 - image * fine) | (int)((unsigned)(int)image << 10), (int)((unsigned)(int)span << 16));
 }
 
 // Load tetrahedron s of cube (ci, cj, ck) and set the walk to the first finest node of its
-// bounding box.  False if a coordinate is not finite (or 2^21 boxes and more away, where float32
-// holds no position): nothing to walk.
+// bounding box.  False if there is nothing to walk (exact_nodes).
 __device__ __forceinline__ bool walk_start(const DepositParams &P, int64_t ci, int64_t cj, int64_t ck, int s,
                                            LeafWalk &w)
 {
     lattice_positions(P, ci, cj, ck, s, w.x);
-    w.shifts = 0;
-    if (may_shift(P, w.x)) {
-#pragma unroll
-        for (int q = 1; q < 4; ++q)
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                const int h = image_shift(P, w.x[q][a], w.x[0][a]);
-                w.shifts |= (unsigned)(h < 0 ? 2 : h) << (2 * (3 * (q - 1) + a));
-            }
-    }
-    const double fine = (double)P.fine, scale = fine / P.box, inv_fine = 1.0 / fine;
+    w.shifts = tet_shift_bits(P, w.x);
+    const float to_node = (float)((double)P.fine / P.box);
     bool ok = true;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        double mn, mx;
-        if (w.shifts == 0) {
-            mn = (double)fminf(fminf(w.x[0][a], w.x[1][a]), fminf(w.x[2][a], w.x[3][a]));
-            mx = (double)fmaxf(fmaxf(w.x[0][a], w.x[1][a]), fmaxf(w.x[2][a], w.x[3][a]));
+        const float mn = fminf(fminf(w.x[0][a], w.x[1][a]), fminf(w.x[2][a], w.x[3][a])) * to_node;
+        const float mx = fmaxf(fmaxf(w.x[0][a], w.x[1][a]), fmaxf(w.x[2][a], w.x[3][a])) * to_node;
+        const float f0 = floorf(mn), f1 = floorf(mx);
+        // the two products' rounding is below 2e-7 of them
+        const float margin = 1e-6f * (1.f + fmaxf(fabsf(mn), fabsf(mx)));
+        const bool sure = w.shifts == 0 && margin < 0.1f && fminf(mn - f0, mx - f1) > margin &&
+                          fmaxf(mn - f0, mx - f1) < 1.f - margin;
+        if (sure) {
+            const int n0 = (int)f0, n1 = (int)f1;
+            w.first[a] = (n0 & ((int)P.fine - 1)) | (int)((unsigned)(n0 >> P.max_level) << 10);
+            w.at[a] = (unsigned)(n1 - n0) << 16;
+            ok = ok && n1 - n0 < 65535;
         } else {
-            mn = mx = (double)w.x[0][a];
-#pragma unroll
-            for (int q = 1; q < 4; ++q) {
-                const double u = (double)w.x[q][a] + (double)walk_shift(w.shifts, q, a) * P.box;
-                mn = fmin(mn, u);
-                mx = fmax(mx, u);
-            }
+            const int2 n = exact_nodes(P, w.shifts, a, w.x[0][a], w.x[1][a], w.x[2][a], w.x[3][a]);
+            w.first[a] = n.x;
+            w.at[a] = (unsigned)n.y;
+            ok = ok && n.y != -1;
         }
-        const double f0 = floor(mn * scale), f1 = floor(mx * scale);
-        const double image = floor(f0 * inv_fine);  // exact: the number of finest nodes is a power of two
-        const double span = f1 - f0;
-        ok = ok && fabs(image) < 2097152.0 && span < 65535.0;
-        w.first[a] = (int)(f0 - image * fine) | (int)((unsigned)(int)image << 10);
-        w.at[a] = (unsigned)(int)span << 16;
     }
     return ok;
 }
@@ -439,7 +438,7 @@ __device__ __forceinline__ void tet_shifts(unsigned shifts, int (&k)[4][3])
 #pragma unroll
     for (int q = 0; q < 4; ++q)
 #pragma unroll
-        for (int a = 0; a < 3; ++a) k[q][a] = walk_shift(shifts, q, a);
+        for (int a = 0; a < 3; ++a) k[q][a] = shift_of(shifts, q, a);
 }
 __device__ __noinline__ double walk_det6(const DepositParams &P, WalkTet t)
 {
@@ -478,7 +477,7 @@ __device__ __forceinline__ void walk_grid(const DepositParams &P, const LeafWalk
         for (int q = 1; q < 4; ++q)
 #pragma unroll
             for (int a = 0; a < 3; ++a)
-                c[q][a] = fmaf(w.x[q][a], sf, (float)((long long)walk_shift(w.shifts, q, a) * g - base[a]));
+                c[q][a] = fmaf(w.x[q][a], sf, (float)((long long)shift_of(w.shifts, q, a) * g - base[a]));
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) v[q] = mk<float>(c[q][0], c[q][1], c[q][2]);
@@ -493,7 +492,10 @@ __device__ __forceinline__ void walk_grid(const DepositParams &P, const LeafWalk
 // take theirs, whichever tetrahedron or leaf they are at, so that a round's 32 records are full
 // until the item's tetrahedra run out.  (Rows of cubes cross leaf blocks, so the lanes of a warp
 // need different numbers of rounds for the same tetrahedron of their cubes: 256^3 octree 294 ->
-// 277 ms, with collapsed regions 345 -> 300 ms, the guarded clips' gain included.)
+// 277 ms, with collapsed regions 345 -> 300 ms, the guarded clips' gain included.)  The warps of an
+// SM compete for its instruction cache, so the steps that few tetrahedra take (periodic shifts,
+// nodes within float32 rounding of a boundary, degenerate ones) are out of line: 268 -> 261 ms,
+// 291 -> 286 ms.
 template <bool STATS, int MINB, Acc A, int PASS>
 __global__ void __launch_bounds__(128, MINB) k_oct_warp(const DepositParams P)
 {
@@ -527,14 +529,14 @@ __global__ void __launch_bounds__(128, MINB) k_oct_warp(const DepositParams P)
                 s_end = s + 1;
             }
         } else {
-            const unsigned parts = 6u / (unsigned)P.subs;  // items per group of cubes
-            const int64_t u = (int64_t)(item / parts) * per + lane;
+            const bool whole = P.subs == 6;  // an item takes all six tetrahedra of its cubes, or one
+            const int64_t u = (int64_t)(whole ? item : item / 6) * per + lane;
             if (lane < per && u < P.n_units) {
                 cube = P.src == SRC_CUBE_LIST ? P.cube_ids[u] : u;
                 if (cube < 0 || cube >= P.nc[0] * P.nc[1] * P.nc[2]) {
                     set_error(P.ws, 3, (int)(u & 0x7fffffff));
                 } else {
-                    s = (int)(item % parts) * P.subs;
+                    s = whole ? 0 : (int)(item % 6);
                     s_end = s + P.subs;
                 }
             }
@@ -549,8 +551,13 @@ __global__ void __launch_bounds__(128, MINB) k_oct_warp(const DepositParams P)
             bool to_list = false;  // the FP32 pass: this tetrahedron's first guarded pair
             int leaf = 0, level = 0;
             int64_t org64[3];
-            bool hit = walk_next(P, w, leaf, level, org64);
-            while (!hit && s < s_end) {  // the next tetrahedron (its first node always is a pair)
+            // the next pair: of this tetrahedron, or the first one of the lane's next tetrahedron
+            // (whose first node always is a pair)
+            bool hit = false;
+#pragma unroll 1
+            for (;;) {
+                hit = walk_next(P, w, leaf, level, org64);
+                if (hit || s >= s_end) break;
                 int64_t ci, cj, ck;
                 cube_coords(P, cube, ci, cj, ck);
                 const bool ok = walk_start(P, ci, cj, ck, s, w);
@@ -563,9 +570,7 @@ __global__ void __launch_bounds__(128, MINB) k_oct_warp(const DepositParams P)
                 ++s;
                 fresh = true;
                 noted = false;
-                if (ok) {
-                    hit = walk_next(P, w, leaf, level, org64);
-                } else {
+                if (!ok) {
                     walk_end(w);
                     set_error(P.ws, 4, lane);
                 }
@@ -577,10 +582,10 @@ __global__ void __launch_bounds__(128, MINB) k_oct_warp(const DepositParams P)
                 TetSetup<float> ts;
                 const bool swapped = tet_setup<float>(v, ts);
                 const bool guard = !(ts.kappa <= P.kappa_max);
-                // Exactly degenerate tetrahedra go to the cell of their centroid, once.  A
-                // well-conditioned one cannot be degenerate: its rounded volume is right to 1%
+                // Exactly degenerate tetrahedra go to the cell of their centroid, once.  Up to kappa
+                // = 1e4 a tetrahedron cannot be degenerate: its rounded volume is right to 1%
                 bool degenerate = false;
-                if (fresh && !(ts.kappa <= fminf(P.kappa_max, 1e4f))) {
+                if (fresh && !(ts.kappa <= 1e4f)) {
                     if (walk_det6(P, walk_tet(w)) == 0.0) {
                         degenerate = true;
                         walk_end(w);  // no further leaf
