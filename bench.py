@@ -777,7 +777,8 @@ def run_precision(args, pse, dev, stream, standalone=True):
                    "h2d_bytes_per_step": int(pos_host.nbytes), "d2h_bytes_per_step": int(out.numel() * 8)}}
     if not args.no_baseline:
         bms = _timed(lambda: pse.deposit_uniform(pos, n, g, out=out, workspace=ws, precision=pse.PSE_FP64_PLAIN,
-                                                 schedule=pse.PSE_THREAD_PER_TET), 1, 1, flush, stream)[0]
+                                                 schedule=pse.PSE_THREAD_PER_TET, tuning={"thread_fp64": 1}),
+                     1, 1, flush, stream)[0]
         ref64 = out.cpu().numpy()
         base = {"tets_per_s": n_tets / (bms * 1e-3), "ms_per_step": bms, "speedup": bms / ms,
                 "error_of_timed_arm": cell_errors(fast_grid, ref64)}

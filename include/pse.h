@@ -76,7 +76,8 @@ extern "C" {
                                   end of the call (needs accumulate = 0) */
 
 /* schedule (pse_deposit_opts.schedule) */
-#define PSE_THREAD_PER_TET 0    /* one thread per tetrahedron (the plain baseline) */
+#define PSE_THREAD_PER_TET 0    /* one thread per tetrahedron (the plain baseline; see
+                                   pse_tuning.thread_fp64 for PSE_FP64_PLAIN) */
 #define PSE_WARP_COOPERATIVE 1  /* one warp per batch of tetrahedra, lanes over (tet, cell) pairs */
 #define PSE_BINNED_PERSISTENT 2 /* size-binned persistent kernel: a bin pass queues every tetrahedron whose
                                    bounding box exceeds pse_tuning.split_cells; one persistent kernel
@@ -183,7 +184,11 @@ typedef struct pse_tuning {
                                 guarded pass visits only them; when more are guarded it scans every
                                 tetrahedron again.  0: the full list; > 0: a smaller capacity; < 0: no
                                 list (always scan again).  Results are the same either way. */
-    int32_t reserved[4];
+    int32_t thread_fp64;     /* PSE_FP64_PLAIN on uniform grids: 1 = one thread per tetrahedron and a clip
+                                per cell in every call (the plain baseline); 0 = calls without h_stats
+                                take the warp-cooperative float64 column clip instead: the same masses
+                                to float64 rounding */
+    int32_t reserved[3];
 } pse_tuning;
 
 /*

@@ -345,7 +345,10 @@ int run_deposit(pse::DepositParams &p, const pse_deposit_opts &o, int64_t cells,
                                            bps, s);
             if (e != cudaSuccess) return cuda_fail(e, "octree deposit launch");
         } else {
-            if (o.schedule == PSE_THREAD_PER_TET) e = pse::launch_thread_per_tet(q, o.precision == PSE_FP64_PLAIN, stats, s);
+            // float64: the column clip, unless the call counts cells (the thread kernel's counters
+            // are per cell) or asks for the thread kernel
+            if (o.precision == PSE_FP64_PLAIN && !stats && !(tu && tu->thread_fp64)) e = pse::launch_warp_plain(q, s);
+            else if (o.schedule == PSE_THREAD_PER_TET) e = pse::launch_thread_per_tet(q, o.precision == PSE_FP64_PLAIN, stats, s);
             else if (o.schedule == PSE_WARP_PER_TET) e = pse::launch_warp_per_tet(q, stats, s);
             else if (binned) e = pse::launch_binned(q, stats, bps, s);
             else e = pse::launch_warp_coop(q, stats, bps, s);

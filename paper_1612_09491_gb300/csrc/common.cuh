@@ -512,6 +512,7 @@ struct GuardSmem {
     double2 slots[21][32];  // each lane's 7 edge slots, 3 double2 each
     double v[12][32];       // exact vertices, positively oriented
     double tol[32];         // classification tolerance of the clip (f64_tolerance)
+    double rho[32];         // the plain float64 path: 6 m_t / |6V|
 };
 
 constexpr int kQBits = 19;  // per-axis cell offset bits in a queue entry
@@ -873,7 +874,7 @@ constexpr int kRunsPerRound = 16;
 // thread would, so the sums are the same bit for bit.  Measured (one GB300, before -> after):
 // 128^3 onto 256^3 45.2 -> 33.8 ms, 48^3 onto 384^3 46.5 -> 31.0 ms, 256^3 octree with collapsed
 // regions 412 -> 345 ms, shell-crossed 128^3 octree (FP64 clips) 233 -> 141 ms.
-template <bool STATS, bool OCT, Acc A, class T>
+template <bool STATS, bool OCT, Acc A, class T, bool F64RHO>
 __device__ __forceinline__ void job_round(const DepositParams &P, WarpSmem *S, int lane, int &head, int &qn, int &jobs,
                                           Counters &cnt)
 {
@@ -1062,8 +1063,10 @@ __device__ __forceinline__ void job_round(const DepositParams &P, WarpSmem *S, i
             }
             if (vol > T(0)) {
                 if (STATS) cnt.u[ST_OVERLAPPED]++;
-                const float rho = S->rho[t];
-                const double m = (sizeof(T) == sizeof(float)) ? (double)(rho * (float)vol) : (double)rho * vol;
+                double m;
+                if constexpr (sizeof(T) == sizeof(float)) m = (double)(S->rho[t] * (float)vol);
+                else if constexpr (F64RHO) m = guard_smem(S)->rho[t] * vol;
+                else m = (double)S->rho[t] * vol;
                 cnt.add_dep(m);
                 if (!deposit_pair<OCT, A>(P, S, t, ex, ey, ez, m) && STATS) cnt.dropped += m;
             }
@@ -1121,6 +1124,14 @@ __device__ __forceinline__ int64_t listed_guarded(const DepositParams &P)
     return c > (unsigned long long)P.guard_cap ? -1 : (int64_t)c;
 }
 
+// 6 m_t / |6V| of record t: float32, or float64 in the plain float64 path (F64RHO).
+template <bool F64RHO>
+__device__ __forceinline__ auto record_rho(WarpSmem *S, int t)
+{
+    if constexpr (F64RHO) return guard_smem(S)->rho[t];
+    else return S->rho[t];
+}
+
 // Inclusive prefix of the lanes' pair counts into S->start (exclusive) and their total.
 __device__ __forceinline__ int pair_prefix(WarpSmem *S, int lane, int npairs)
 {
@@ -1149,7 +1160,7 @@ __device__ __forceinline__ int pair_record(const WarpSmem *S, int idx)
 // run count; skip: the first run of the records, for pieces of a split tetrahedron), 32 per
 // step: classify; deposit the cells of "inside" runs; queue the partial runs with their clip
 // frame and the faces that reach their column, and clip 32 faces at a time.
-template <bool STATS, bool OCT, Acc A, class T>
+template <bool STATS, bool OCT, Acc A, class T, bool F64RHO = false>
 __device__ __forceinline__ void coop_runs(const DepositParams &P, WarpSmem *S, int lane, int npairs, int skip,
                                           Counters &cnt)
 {
@@ -1176,7 +1187,7 @@ __device__ __forceinline__ void coop_runs(const DepositParams &P, WarpSmem *S, i
                       cz = C == 2 ? lc : (C == 0 ? lb : la);
             const int cls = classify_run(S, t, C, (float)cx, (float)cy, (float)cz, kw);
             if (cls == CELL_INSIDE) {
-                const double m = (double)S->rho[t];
+                const double m = (double)record_rho<F64RHO>(S, t);
                 for (int j = 0; j < kw; ++j) {
                     cnt.add_dep(m);
                     if (!deposit_pair<OCT, A>(P, S, t, cx + (C == 0 ? j : 0), cy + (C == 1 ? j : 0),
@@ -1229,7 +1240,7 @@ __device__ __forceinline__ void coop_runs(const DepositParams &P, WarpSmem *S, i
         __syncwarp();
         const bool last = b0 + 32 >= total;
 #pragma unroll 1
-        while (jobs >= 32 || (last && qn > 0)) job_round<STATS, OCT, A, T>(P, S, lane, head, qn, jobs, cnt);
+        while (jobs >= 32 || (last && qn > 0)) job_round<STATS, OCT, A, T, F64RHO>(P, S, lane, head, qn, jobs, cnt);
     }
     cnt.fold_dep();
 }

@@ -3,6 +3,8 @@
 //  * k_thread_per_tet<T>: one thread per tetrahedron walks its bounding-box cells,
 //    classifies each, clips the partial ones and adds m_t V_ov/|V_t| with a global
 //    float64 atomic.  With T = double this is the plain FP64 baseline.
+//  * k_warp_plain: the same results in float64 by the warp-cooperative column clip (calls without
+//    statistics).
 //  * k_warp_coop (coop.cuh): the warp-cooperative FP32 kernel; this file instantiates
 //    its FP64-reduction variants, deposit_comp.cu the compensated-FP32 ones.
 //  * k_warp_per_tet: the paper's warp-per-tetrahedron design (Sec. 6.2), a baseline.
@@ -122,6 +124,159 @@ __global__ void __launch_bounds__(128) k_thread_per_tet(const DepositParams P)
     }
     if (STATS) cnt.flush(P.ws);
     if (P.fixup || STATS) cnt.flush_mass(P, P.ws);
+}
+
+// ---------------------------------------------------------------------------
+// every step in float64, by the warp-cooperative column clip
+// ---------------------------------------------------------------------------
+// Cell by cell for a tetrahedron that the run queue cannot hold (2^25 cells and more): its own
+// thread, as k_thread_per_tet does.
+__device__ __noinline__ void plain_cells(const DepositParams &P, TetSetup<double> ts, int bx, int by, int bz, double rho)
+{
+    for (int iz = 0; iz < ts.dim[2]; ++iz)
+        for (int iy = 0; iy < ts.dim[1]; ++iy)
+            for (int ix = 0; ix < ts.dim[0]; ++ix) {
+                const int cx = ts.lo[0] + ix, cy = ts.lo[1] + iy, cz = ts.lo[2] + iz;
+                const int cls = classify_cell<double>(ts.n, ts.e, ts.pos, ts.neg, (double)cx, (double)cy, (double)cz);
+                double vol = cls == CELL_INSIDE ? 1.0 : 0.0;
+                if (cls == CELL_PARTIAL) {
+                    P3<double> p[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        p[q] = mk<double>(ts.v[q].x - cx, ts.v[q].y - cy, ts.v[q].z - cz);
+                    double err;
+                    vol = overlap_volume_ax<double>(p, ts.n, ts.axis, ts.lx, ts.ly, err);
+                }
+                if (vol > 0.0) deposit_cell<Acc::F64>(P, bx + cx, by + cy, bz + cz, rho * vol);
+            }
+}
+__device__ __noinline__ void plain_large(const DepositParams &P, double x0, double y0, double z0, double x1, double y1,
+                                         double z1, double x2, double y2, double z2, double x3, double y3, double z3,
+                                         int bx, int by, int bz, double m_t)
+{
+    P3<double> v[4] = {mk<double>(x0, y0, z0), mk<double>(x1, y1, z1), mk<double>(x2, y2, z2), mk<double>(x3, y3, z3)};
+    TetSetup<double> ts;
+    tet_setup<double>(v, ts);
+    plain_cells(P, ts, bx, by, bz, 6.0 * m_t / ts.vol6);
+}
+
+// PSE_FP64_PLAIN without statistics: the warp-cooperative schedule with the guarded pass's
+// float64 column clip for every tetrahedron.  Vertices, volume, bounding box and deposits are
+// float64; the float32 copies in the record only choose work: the clip's axis, frame and faces,
+// and the runs that lie wholly inside or outside by a margin above their rounding (1e-6 (L + 1)^3
+// on the plane values for an extent of L cells); everything else is clipped.
+//
+// The float64 pipe bounds both this and the thread-per-tetrahedron kernel (16 cycles a warp
+// instruction).  That kernel clips cell by cell with 9 of 32 lanes active; here one clip serves
+// two cells, with 2.5 times fewer float64 operations, and the lanes are full: 48^3 on 96^3 213 ->
+// 17.6 ms, the masses equal to 3e-16 (norm).
+__global__ void __launch_bounds__(kCoopThreads, 2) k_warp_plain(const DepositParams P)
+{
+    WarpSmem *S = warp_smem(true);
+    GuardSmem *G = guard_smem(S);
+    const int lane = threadIdx.x & 31;
+    Counters cnt;
+    cnt.zero_mass();
+    for (;;) {
+        unsigned long long item = 0;
+        if (lane == 0) item = atomicAdd(&P.ws->work_counter, 1ull);
+        item = __shfl_sync(kFull, item, 0);
+        if ((int64_t)item >= P.n_items) break;
+        int64_t g = (int64_t)item, ci = 0, cj = 0, ck = 0;
+        int s = 0;
+        if (P.src != SRC_TETS) {
+            s = (int)(item % 6);
+            g = (int64_t)(item / 6);
+        }
+        const int64_t u = g * P.group + lane;
+        bool have = lane < P.group && u < P.n_units;
+        if (have && P.src != SRC_TETS && !cube_of_unit(P, u, ci, cj, ck)) {
+            set_error(P.ws, 3, (int)(u & 0x7fffffff));
+            have = false;
+        }
+        int npairs = 0;
+        if (have) {
+            P3<double> v[4];
+            int base[3];
+            double m_t;
+            if (P.src == SRC_TETS) {
+                explicit_tet<double>(P, u, v, base);
+                m_t = P.tet_mass[u];
+            } else {
+                lattice_tet<double>(P, ci, cj, ck, s, v, base);
+                m_t = P.m_tet;
+            }
+            const double d6 = det6(v), vol6 = fabs(d6);
+            if (d6 < 0.0) {
+                const P3<double> t = v[1];
+                v[1] = v[2];
+                v[2] = t;
+            }
+            TetSetup<float> ts;  // of the float32 vertices; its cell range replaced by the float64 one
+            P3<float> vf[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) vf[q] = mk<float>((float)v[q].x, (float)v[q].y, (float)v[q].z);
+            {
+                const double mnx = fmin(fmin(v[0].x, v[1].x), fmin(v[2].x, v[3].x)), mxx = fmax(fmax(v[0].x, v[1].x), fmax(v[2].x, v[3].x));
+                const double mny = fmin(fmin(v[0].y, v[1].y), fmin(v[2].y, v[3].y)), mxy = fmax(fmax(v[0].y, v[1].y), fmax(v[2].y, v[3].y));
+                const double mnz = fmin(fmin(v[0].z, v[1].z), fmin(v[2].z, v[3].z)), mxz = fmax(fmax(v[0].z, v[1].z), fmax(v[2].z, v[3].z));
+                P3<float> w[4] = {vf[0], vf[1], vf[2], vf[3]};
+                tet_setup<float>(w, ts);
+                const double big = 16777216.0;
+                const bool fin = d6 == d6 && mnx > -big && mxx < big && mny > -big && mxy < big && mnz > -big && mxz < big;
+                ts.lo[0] = fin ? (int)floor(mnx) : 0;
+                ts.lo[1] = fin ? (int)floor(mny) : 0;
+                ts.lo[2] = fin ? (int)floor(mnz) : 0;
+                ts.dim[0] = fin ? (int)floor(mxx) - ts.lo[0] + 1 : 0;
+                ts.dim[1] = fin ? (int)floor(mxy) - ts.lo[1] + 1 : 0;
+                ts.dim[2] = fin ? (int)floor(mxz) - ts.lo[2] + 1 : 0;
+            }
+            const int64_t ncell = (int64_t)ts.dim[0] * ts.dim[1] * ts.dim[2];
+            if (!tet_ok(base, ts)) {
+                set_error(P.ws, 4, lane);
+            } else if (vol6 == 0.0) {
+                int c[3];
+                centroid_cell(v, c);
+                deposit_cell<Acc::F64>(P, base[0] + c[0], base[1] + c[1], base[2] + c[2], m_t);
+            } else if (ncell == 1) {
+                deposit_cell<Acc::F64>(P, base[0] + ts.lo[0], base[1] + ts.lo[1], base[2] + ts.lo[2], m_t);
+            } else if (ncell > (int64_t)(1 << 25) || !dims_fit_queue(ts.dim)) {
+                plain_large(P, v[0].x, v[0].y, v[0].z, v[1].x, v[1].y, v[1].z, v[2].x, v[2].y, v[2].z, v[3].x, v[3].y,
+                            v[3].z, base[0], base[1], base[2], m_t);
+            } else {
+                npairs = (int)run_count(ts.dim, ts.axis);
+                const float l1 = 1.f + (float)max(ts.dim[0], max(ts.dim[1], ts.dim[2])), margin = 1e-6f * l1 * l1 * l1;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    S->v[3 * q][lane] = vf[q].x;
+                    S->v[3 * q + 1][lane] = vf[q].y;
+                    S->v[3 * q + 2][lane] = vf[q].z;
+                    G->v[3 * q][lane] = v[q].x;
+                    G->v[3 * q + 1][lane] = v[q].y;
+                    G->v[3 * q + 2][lane] = v[q].z;
+                    S->n[3 * q][lane] = ts.n[q].x;
+                    S->n[3 * q + 1][lane] = ts.n[q].y;
+                    S->n[3 * q + 2][lane] = ts.n[q].z;
+                    S->e[q][lane] = ts.e[q];
+                    S->pos[q][lane] = ts.pos[q] + margin;
+                    S->neg[q][lane] = ts.neg[q] - margin;
+                }
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    S->lo[a][lane] = ts.lo[a];
+                    S->dim[a][lane] = ts.dim[a];
+                    S->base[a][lane] = base[a];
+                }
+                S->lx[lane] = ts.lx;
+                S->ly[lane] = ts.ly;
+                S->axis[lane] = ts.axis;
+                G->rho[lane] = 6.0 * m_t / vol6;
+                G->tol[lane] = f64_tolerance((double)(ts.dim[0] + ts.dim[1] + ts.dim[2]));
+            }
+        }
+        coop_runs<false, false, Acc::F64, double, true>(P, S, lane, npairs, 0, cnt);
+        __syncwarp();
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -409,6 +564,19 @@ cudaError_t launch_thread_per_tet(const DepositParams &p, bool fp64, bool stats,
         else k_thread_per_tet<float, false><<<(unsigned)blocks, threads, 0, st>>>(p);
     }
     return cudaGetLastError();
+}
+
+cudaError_t launch_warp_plain(const DepositParams &p, cudaStream_t st)
+{
+    const void *k = (const void *)k_warp_plain;
+    const size_t smem = warp_smem_bytes(kCoopThreads / 32, true);
+    cudaError_t err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (err != cudaSuccess) return err;
+    int64_t blocks = persistent_blocks(k, kCoopThreads, smem);
+    const int64_t need = (p.n_items + kCoopThreads / 32 - 1) / (kCoopThreads / 32);
+    if (need < blocks) blocks = need < 1 ? 1 : need;
+    void *args[] = {const_cast<DepositParams *>(&p)};
+    return cudaLaunchKernel(k, dim3((unsigned)blocks), dim3(kCoopThreads), args, smem, st);
 }
 
 cudaError_t launch_warp_coop(const DepositParams &p, bool stats, int blocks_per_sm, cudaStream_t st)

@@ -126,6 +126,8 @@ void set_last_error(const char *msg);
 
 // launchers (deposit.cu)
 cudaError_t launch_thread_per_tet(const DepositParams &p, bool fp64, bool stats, cudaStream_t st);
+// float64, without statistics: the warp-cooperative column clip
+cudaError_t launch_warp_plain(const DepositParams &p, cudaStream_t st);
 cudaError_t launch_warp_coop(const DepositParams &p, bool stats, int blocks_per_sm, cudaStream_t st);
 cudaError_t launch_binned(const DepositParams &p, bool stats, int blocks_per_sm, cudaStream_t st);
 cudaError_t launch_warp_per_tet(const DepositParams &p, bool stats, cudaStream_t st);
