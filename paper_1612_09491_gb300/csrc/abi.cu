@@ -161,10 +161,11 @@ void fill_grid(pse::DepositParams &p, const int64_t grid_n[3], double box)
 
 // The work items of the warp kernels.  An item is one warp's batch of up to 32 tetrahedra: the
 // same Kuhn tetrahedron of 32 consecutive cubes (octree: all six, one after another, while there
-// are many items), or 32 tetrahedra of an explicit set.  Small deposits take fewer cubes an item,
-// so that every warp the GPU holds (16 on each of 152 SMs) gets one.  (Before, an item was a row
-// segment of 32 cubes with all six tetrahedra: 16^3 on 32^3 0.86 -> 0.46 ms, 32^3 on 64^3 0.92 ->
-// 0.56 ms, 48^3 on 384^3, whose rows fill three quarters of a warp, 31.0 -> 18.3 ms, 256^3 on
+// are many items), or 32 tetrahedra of an explicit set.  The items are made as large as lets them
+// fill a whole number of waves of the warps that the GPU holds (16 on each of 152 SMs), which
+// matters for small deposits: 16^3 on 32^3 170 us with 8 cubes an item (1.3 waves), 154 us with 11
+// (one wave); 32^3 on 64^3 549 -> 536 us.  (Before, an item was a row segment of 32 cubes with all
+// six tetrahedra: 16^3 on 32^3 0.86 ms, 32^3 on 64^3 0.92 ms, 48^3 on 384^3, whose rows fill three quarters of a warp, 31.0 -> 18.3 ms, 256^3 on
 // 128^3 64.7 -> 56.4 ms.)
 // The FP32 pass on a uniform grid paces its blocks (coop.cuh) up to this many cells a cube.  160^3
 // cubes, unpaced and paced: 0.5 cells 18.4 and 16.7 ms, 1 cell 21.7 and 20.5, 2 cells 27.5 and
@@ -175,8 +176,8 @@ void set_items(pse::DepositParams &p)
 {
     constexpr int64_t kWarps = 152 * 16;
     const int64_t nsub = p.src == pse::SRC_TETS ? 1 : 6;
-    p.group = 32;
-    while (p.group > 8 && (p.n_units + p.group - 1) / p.group * nsub < 2 * kWarps) p.group /= 2;
+    const int64_t tets = p.n_units * nsub, waves = (tets + 32 * kWarps - 1) / (32 * kWarps);
+    p.group = tets > 0 ? (int)((tets + kWarps * waves - 1) / (kWarps * waves)) : 32;
     const int64_t groups = (p.n_units + p.group - 1) / p.group;
     p.subs = (p.leaves && groups >= 4 * kWarps) ? 6 : 1;
     p.n_items = groups * (nsub / (p.leaves ? p.subs : 1));
