@@ -167,12 +167,12 @@ void fill_grid(pse::DepositParams &p, const int64_t grid_n[3], double box)
 // (one wave); 32^3 on 64^3 549 -> 536 us.  (Before, an item was a row segment of 32 cubes with all
 // six tetrahedra: 16^3 on 32^3 0.86 ms, 32^3 on 64^3 0.92 ms, 48^3 on 384^3, whose rows fill three quarters of a warp, 31.0 -> 18.3 ms, 256^3 on
 // 128^3 64.7 -> 56.4 ms.)
-// The FP32 pass on a uniform grid paces its blocks (coop.cuh) up to this many cells a cube.  160^3
+// The FP32 pass paces its blocks (coop.cuh) up to this many output cells a cube.  160^3
 // cubes, unpaced and paced: 0.5 cells 18.4 and 16.7 ms, 1 cell 21.7 and 20.5, 2 cells 27.5 and
 // 27.4, 4 cells 38.8 and 39.7.
 constexpr double kPaceCells = 2.0;
 
-void set_items(pse::DepositParams &p)
+void set_items(pse::DepositParams &p, int64_t cells)
 {
     constexpr int64_t kWarps = 152 * 16;
     const int64_t nsub = p.src == pse::SRC_TETS ? 1 : 6;
@@ -182,9 +182,7 @@ void set_items(pse::DepositParams &p)
     p.subs = (p.leaves && groups >= 4 * kWarps) ? 6 : 1;
     p.n_items = groups * (nsub / (p.leaves ? p.subs : 1));
     if (p.slab) return;  // a slab keeps the whole lattice's choice
-    p.pace = (!p.leaves && p.src != pse::SRC_TETS &&
-              (double)p.g[0] * (double)p.g[1] * (double)p.g[2] <= kPaceCells * (double)p.nc[0] * (double)p.nc[1] *
-                                                                      (double)p.nc[2])
+    p.pace = (p.src != pse::SRC_TETS && (double)cells <= kPaceCells * (double)p.nc[0] * (double)p.nc[1] * (double)p.nc[2])
                  ? 1 : 0;
 }
 
@@ -241,7 +239,7 @@ int stream_slabs(const float *h_pos, const pse::DepositParams &base, int64_t sla
         p.nc[2] = k1 - k0;
         p.src = pse::SRC_LATTICE;
         p.n_units = p.nc[0] * p.nc[1] * p.nc[2];
-        set_items(p);
+        set_items(p, 0);
         rc = per_slab(p, st);
         if (rc != PSE_OK) break;
         e = cudaEventRecord(freed[b], st);
@@ -335,7 +333,7 @@ int run_deposit(pse::DepositParams &p, const pse_deposit_opts &o, int64_t cells,
     const bool comp = o.precision == PSE_FP32_COMPENSATED;
     p.comp = comp ? 1 : 0;
     const int bps = (tu && tu->blocks_per_sm > 0) ? tu->blocks_per_sm : kDefaultBlocksPerSm;
-    set_items(p);
+    set_items(p, cells);
 
     // the kernels of one deposit pass over the tetrahedra of q, on stream s
     auto launch = [&](const pse::DepositParams &q, cudaStream_t s) -> int {

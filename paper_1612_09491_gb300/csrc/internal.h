@@ -83,7 +83,7 @@ struct DepositParams {
     // scheduling
     int64_t n_items;
     int32_t group;             // cubes (tetrahedra of SRC_TETS) that one work item of the warp kernels takes
-    int32_t pace;              // uniform FP32 pass: 1 = the warps of a block start their items together
+    int32_t pace;              // FP32 pass: 1 = the warps of a block start their items together
     int32_t subs;              // octree: Kuhn tetrahedra of each cube that an item takes (1 or 6); else 1
     Workspace *ws;
     // binned schedule: tetrahedra whose bounding box has more than split_cells cells are

@@ -496,7 +496,11 @@ __device__ __forceinline__ void walk_grid(const DepositParams &P, const LeafWalk
 // SM compete for its instruction cache, so the steps that few tetrahedra take (periodic shifts,
 // nodes within float32 rounding of a boundary, degenerate ones) are out of line: 268 -> 261 ms,
 // 291 -> 286 ms.
-template <bool STATS, int MINB, Acc A, int PASS>
+//
+// PACE (DepositParams::pace): the warps of a block set their records up together, as in
+// k_warp_coop; a variant of its own, because the test alone costs the other octree deposits 0.5%
+// (shell-crossed 128^3: 81.0 -> 79.2 ms).
+template <bool STATS, int MINB, Acc A, int PASS, bool PACE = false>
 __global__ void __launch_bounds__(128, MINB) k_oct_warp(const DepositParams P)
 {
     constexpr bool FIRST = PASS == kPassFp32;
@@ -512,11 +516,21 @@ __global__ void __launch_bounds__(128, MINB) k_oct_warp(const DepositParams P)
     const int per = LIST ? listed_per_item(listed) : P.group;
     const int64_t n_items = LIST ? (listed + per - 1) / per : P.n_items;
 
+    __shared__ unsigned long long block_item;
     for (;;) {
         unsigned long long item = 0;
-        if (lane == 0) item = atomicAdd(FIRST ? &P.ws->work_counter : &P.ws->work_counter2, 1ull);
-        item = __shfl_sync(kFull, item, 0);
-        if ((int64_t)item >= n_items) break;
+        if constexpr (PACE) {
+            __syncthreads();
+            if (threadIdx.x == 0) block_item = atomicAdd(&P.ws->work_counter, (unsigned long long)(blockDim.x >> 5));
+            __syncthreads();
+            item = block_item;
+            if ((int64_t)item >= n_items) break;  // the same for the whole block
+            item += threadIdx.x >> 5;             // (items past the last hold no cube)
+        } else {
+            if (lane == 0) item = atomicAdd(FIRST ? &P.ws->work_counter : &P.ws->work_counter2, 1ull);
+            item = __shfl_sync(kFull, item, 0);
+            if ((int64_t)item >= n_items) break;
+        }
         // this lane's cube and its tetrahedra s .. s_end-1
         int64_t cube = 0;
         int s = 0, s_end = 0;
@@ -546,7 +560,13 @@ __global__ void __launch_bounds__(128, MINB) k_oct_warp(const DepositParams P)
         bool fresh = false;  // the walk's tetrahedron has not met a leaf yet
         bool noted = false;  // ... is on the guarded list
 #pragma unroll 1
-        while (__any_sync(kFull, s < s_end || !walk_done(w))) {
+        for (;;) {
+            const bool left = s < s_end || !walk_done(w);
+            if constexpr (PACE) {
+                if (!__syncthreads_or(left)) break;
+            } else {
+                if (!__any_sync(kFull, left)) break;
+            }
             int npairs = 0;
             bool to_list = false;  // the FP32 pass: this tetrahedron's first guarded pair
             int leaf = 0, level = 0;
@@ -1026,11 +1046,13 @@ cudaError_t launch_oct_pass(const DepositParams &p, bool stats, int blocks_per_s
                    : (stats ? (const void *)k_oct_warp<true, 2, Acc::F64, PASS> : (const void *)k_oct_warp<false, 2, Acc::F64, PASS>);
     } else {
         k = p.comp ? (stats ? (const void *)k_oct_warp<true, 2, Acc::COMP, PASS>
-                      : minb == 4 ? (const void *)k_oct_warp<false, 4, Acc::COMP, PASS>
+                      : minb == 4 ? (p.pace ? (const void *)k_oct_warp<false, 4, Acc::COMP, PASS, true>
+                                            : (const void *)k_oct_warp<false, 4, Acc::COMP, PASS>)
                       : minb == 3 ? (const void *)k_oct_warp<false, 3, Acc::COMP, PASS>
                                   : (const void *)k_oct_warp<false, 2, Acc::COMP, PASS>)
             : (stats ? (const void *)k_oct_warp<true, 2, Acc::F64, PASS>
-               : minb == 4 ? (const void *)k_oct_warp<false, 4, Acc::F64, PASS>
+               : minb == 4 ? (p.pace ? (const void *)k_oct_warp<false, 4, Acc::F64, PASS, true>
+                                     : (const void *)k_oct_warp<false, 4, Acc::F64, PASS>)
                : minb == 3 ? (const void *)k_oct_warp<false, 3, Acc::F64, PASS>
                            : (const void *)k_oct_warp<false, 2, Acc::F64, PASS>);
     }
