@@ -295,19 +295,29 @@ int run_deposit(pse::DepositParams &p, const pse_deposit_opts &o, int64_t cells,
     // streamed: tetrahedron ids (cost-model bitmap) are slab-local
     const int64_t n_tets = streamed ? 6 * p.nc[0] * p.nc[1] * std::min(slab_cubes, p.nc[2])
                                     : (p.src == pse::SRC_TETS) ? p.n_units : 6 * p.n_units;
-    int rc = acquire_ws(d_ws, ws_bytes, st, lease, p.leaves ? octree_ws_bytes(&o) : deposit_ws_bytes(&o, n_tets),
-                        false);
+    size_t need = p.leaves ? octree_ws_bytes(&o) : deposit_ws_bytes(&o, n_tets);
+    // A workspace of the library's own, allocated and freed in this call, leaves out what the call
+    // cannot use: the residual blocks (the warp-per-tetrahedron baseline's) and list entries beyond
+    // the call's tetrahedra.  Mapping 38 MB made up most of a small call that starts on an idle
+    // device: 16^3 on 32^3 without a workspace 0.45 -> 0.37 ms.
+    size_t res_bytes = pse::kResidualBytes, list_bytes = pse::kGuardListBytes;
+    if (d_ws == nullptr && o.schedule != PSE_THREAD_PER_TET && need > 0) {
+        const size_t full = need;
+        if (o.schedule != PSE_WARP_PER_TET || p.leaves) res_bytes = 0;
+        if (n_tets < pse::kGuardListCap) list_bytes = ((size_t)n_tets * 8 + 255) / 256 * 256;
+        need = full - (pse::kResidualBytes - res_bytes) - (pse::kGuardListBytes - list_bytes);
+    }
+    int rc = acquire_ws(d_ws, ws_bytes, st, lease, need, false);
     if (rc != PSE_OK) return rc;
     p.ws = lease.ws;
     if (o.schedule != PSE_THREAD_PER_TET)
         p.vres = reinterpret_cast<float *>(reinterpret_cast<unsigned char *>(lease.ws) + pse::kWorkspaceBytes);
-    unsigned char *const list = reinterpret_cast<unsigned char *>(lease.ws) + pse::kWorkspaceBytes +
-                                pse::kResidualBytes;
-    unsigned char *const after_res = list + pse::kGuardListBytes;
+    unsigned char *const list = reinterpret_cast<unsigned char *>(lease.ws) + pse::kWorkspaceBytes + res_bytes;
+    unsigned char *const after_res = list + list_bytes;
     if (o.schedule != PSE_THREAD_PER_TET) {
-        const int32_t cap = tu ? tu->guard_list_cap : 0;
+        const int64_t cap = tu ? tu->guard_list_cap : 0, room = (int64_t)(list_bytes / 8);
         p.guard_list = reinterpret_cast<int64_t *>(list);
-        p.guard_cap = cap < 0 ? 0 : (cap > 0 && cap < pse::kGuardListCap ? cap : pse::kGuardListCap);
+        p.guard_cap = cap < 0 ? 0 : (cap > 0 && cap < room ? cap : room);
     }
     size_t qbits_len = 0;
     if (binned && o.cost_model) {
