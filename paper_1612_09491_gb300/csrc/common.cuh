@@ -929,7 +929,7 @@ __device__ __forceinline__ void job_round(const DepositParams &P, WarpSmem *S, i
                 const P3<float> a = sub(src.vtx(ia), q), b = sub(src.vtx(ib), q), c = sub(src.vtx(ic), q);
                 const P3<float> nf = src.nrm(f);
                 if (face_meets_column<float>(a, b, c, nf.z, F))
-                    face_run<kRun, float>(a, b, c, nf, F, lane_slots(S, lane, 0.f), fr);
+                    face_run<kRun, float, OCT>(a, b, c, nf, F, lane_slots(S, lane, 0.f), fr);
             } else {
                 // straight into the frame: first cell + q is exact
                 const RecordRun<double> src = record_run<double>(S, t, C, widen<double>(ra.x) + F.qx,
