@@ -705,60 +705,6 @@ __device__ __forceinline__ EdgeSlots<double> lane_slots(WarpSmem *S, int lane, d
     return {&guard_smem(S)->slots[0][lane]};
 }
 
-// The faces of a run that can reach its column [0,1)^2 (bit f), from the projected vertices p
-// (clip frame, relative to the run's first cell) and the signs of the normals' z components
-// (up: bit f set if face f's is positive).  A face is left out when the square lies beyond its
-// bounding box or beyond one of its edges by a margin far above the rounding of the clip, which
-// would then find an empty polygon and add exactly 0, so leaving it out changes no bit: the
-// margins are 2e-3 of a cell plus 4e-6 (m + 1)^2 on the edge functions (m: the largest
-// coordinate), against errors of about 3e-6 m in positions and 1e-6 m^2 in the edge functions;
-// beyond m = 500 every face is kept.  A face seen edge-on, whose sign is rounding, is a segment
-// to within those errors, so either sign is safe.  On the headline workload's tetrahedra this
-// leaves 2.8 of 4 faces a run (3.2 by the bounding boxes alone).
-__device__ __forceinline__ unsigned face_mask(const P3<float> (&p)[4], unsigned up)
-{
-    float m = 0.f;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) m = fmaxf(m, fmaxf(fmaxf(fabsf(p[i].x), fabsf(p[i].y)), fabsf(p[i].z)));
-    if (!(m <= 500.f)) return 15u;
-    const float gap = 2e-3f;
-    bool out[4];
-    {
-        const float lx = fminf(p[0].x, p[1].x), hx = fmaxf(p[0].x, p[1].x), lx2 = fminf(p[2].x, p[3].x),
-                    hx2 = fmaxf(p[2].x, p[3].x);
-        const float ly = fminf(p[0].y, p[1].y), hy = fmaxf(p[0].y, p[1].y), ly2 = fminf(p[2].y, p[3].y),
-                    hy2 = fmaxf(p[2].y, p[3].y);
-#pragma unroll
-        for (int f = 0; f < 4; ++f) {
-            // the face's vertices: the other one of f's pair, and the other pair
-            const P3<float> s = p[f ^ 1];
-            const bool lowpair = f < 2;
-            const float mnx = fminf(s.x, lowpair ? lx2 : lx), mxx = fmaxf(s.x, lowpair ? hx2 : hx);
-            const float mny = fminf(s.y, lowpair ? ly2 : ly), mxy = fmaxf(s.y, lowpair ? hy2 : hy);
-            out[f] = mxx < -gap || mnx > 1.f + gap || mxy < -gap || mny > 1.f + gap;
-        }
-    }
-    // edge i -> j: the square is wholly to its left (L) or right (R)
-    const float eps = 4e-6f * (m + 1.f) * (m + 1.f);
-    bool L[6], R[6];
-    constexpr int ei[6] = {0, 0, 0, 1, 1, 2}, ej[6] = {1, 2, 3, 2, 3, 3};
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        const P3<float> a = p[ei[k]], b = p[ej[k]];
-        const float dx = b.x - a.x, dy = b.y - a.y;
-        const float c = dx * (0.5f - a.y) - dy * (0.5f - a.x);
-        const float r = fmaf(0.5f + gap, fabsf(dx) + fabsf(dy), eps);
-        L[k] = c > r;
-        R[k] = c < -r;
-    }
-    // outward loops (face_vertices): 1-2-3, 0-3-2, 0-1-3, 0-2-1; counter-clockwise when up
-    const bool s0 = (up & 1u) ? (R[3] || R[5] || L[4]) : (L[3] || L[5] || R[4]);
-    const bool s1 = (up & 2u) ? (R[2] || L[5] || L[1]) : (L[2] || R[5] || R[1]);
-    const bool s2 = (up & 4u) ? (R[0] || R[4] || L[2]) : (L[0] || L[4] || R[2]);
-    const bool s3 = (up & 8u) ? (R[1] || L[3] || L[0]) : (L[1] || R[3] || R[0]);
-    return (out[0] || s0 ? 0u : 1u) | (out[1] || s1 ? 0u : 2u) | (out[2] || s2 ? 0u : 4u) | (out[3] || s3 ? 0u : 8u);
-}
-
 // Classify the box of kw cells from cell (cx, cy, cz) along axis C against record t's
 // face planes (classify_cell for kw = 1).
 __device__ __forceinline__ int classify_run(const WarpSmem *S, int t, int C, float cx, float cy, float cz, int kw)

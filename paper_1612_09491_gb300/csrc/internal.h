@@ -69,7 +69,7 @@ struct DepositParams {
     double scale_d[3];         // g_a / box
     float scale_f[3];
     double *out;
-    float *vres;               // warp kernels: kMaxWarpBlocks * 4 residual blocks (see kResidualBytes)
+    float *vres;               // warp-per-tetrahedron baseline: residual blocks (see kResidualBytes)
     // numerics
     float kappa_max;           // FP32 path: tetrahedra with kappa above this clip in float64
     int32_t fixup;             // accumulate mass_target / mass_deposited for the renormalisation
@@ -103,11 +103,10 @@ struct DepositParams {
     int64_t guard_cap;
 };
 
-// warp kernels (every schedule but thread-per-tetrahedron): the float32 rounding residuals
-// of guarded records live in global memory, one [12][32] float block per warp of the
-// grid, right after the Workspace header; their grids are capped at kMaxWarpBlocks blocks
-// of 4 warps (persistent kernels, so the cap only bounds the parallelism).  Keeping them
-// out of shared memory lets 4 blocks of 128 threads share an SM.
+// warp kernels: persistent grids of at most kMaxWarpBlocks blocks (the cap only bounds the
+// parallelism).  The warp-per-tetrahedron baseline keeps the float32 rounding residuals of guarded
+// records in global memory, one [12][32] float block per warp of the grid, right after the
+// Workspace header; the column-clip kernels hold exact vertices in shared memory instead.
 constexpr int kMaxWarpBlocks = 1024;
 constexpr size_t kResidualBytes = (size_t)kMaxWarpBlocks * 4 * 12 * 32 * sizeof(float);
 
