@@ -712,6 +712,14 @@ __device__ __noinline__ int3 exact_node(const DepositParams &P, int64_t ci, int6
     return make_int3(c[0], c[1], c[2]);
 }
 
+// Offset of a corner coordinate from corner 000's at its nearest periodic image.  Out of line: the
+// compiler otherwise evaluates its float64 for every corner (4.9 against 2.5 ms for 256^3).
+__device__ __noinline__ float far_offset(double box, float x, float x0)
+{
+    const double d = (double)x - (double)x0;
+    return (float)(d + (double)((d >= 0.5 * box) ? -1 : ((d < -0.5 * box) ? 1 : 0)) * box);
+}
+
 // One pass over the tetrahedra: per level 0 .. max_level-1, the node that holds the
 // tetrahedron's vertex centroid and the 64-bin log10 histogram bin of its mean edge length
 // in that level's cells.  A lane takes one Lagrangian cube (a warp: 32 neighbouring cubes of a
@@ -725,7 +733,7 @@ __device__ __noinline__ int3 exact_node(const DepositParams &P, int64_t ci, int6
 // the rounding of a boundary is decided by the float64 centroid and the level's own log10.
 // Float32 errors: below 4e-7 of the box and of the position for a centroid, below 2e-5 of a bin
 // for the shifted logarithm; the margins are 2e-6 and 4e-5.  Measured: the 256^3 octree build and
-// deposit 277 -> 270.5 ms.
+// deposit 277 -> 270.5 ms, and 2.4 ms less with far_offset out of line.
 __global__ void __launch_bounds__(256) k_tet_size_hist(const DepositParams P, unsigned *__restrict__ hist)
 {
     __shared__ unsigned sh[64 + 512];  // levels 0 and 1 aggregated per block
@@ -764,8 +772,7 @@ __global__ void __launch_bounds__(256) k_tet_size_hist(const DepositParams P, un
                         x0[a] = x;
                     } else {
                         float d = x - x0[a];
-                        if (P.periodic && !(fabsf(d) < near))
-                            d = (float)(((double)x - (double)x0[a]) + (double)image_shift(P, x, x0[a]) * P.box);
+                        if (P.periodic && !(fabsf(d) < near)) d = far_offset(P.box, x, x0[a]);
                         r[c][a] = d;
                     }
                 }
