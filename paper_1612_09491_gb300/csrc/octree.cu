@@ -604,18 +604,9 @@ __global__ void __launch_bounds__(128, MINB) k_oct_warp(const DepositParams P)
                 const bool guard = !(ts.kappa <= P.kappa_max);
                 // Exactly degenerate tetrahedra go to the cell of their centroid, once.  Up to kappa
                 // = 1e4 a tetrahedron cannot be degenerate: its rounded volume is right to 1%
-                bool degenerate = false;
-                if (fresh && !(ts.kappa <= 1e4f)) {
-                    if (walk_det6(P, walk_tet(w)) == 0.0) {
-                        degenerate = true;
-                        walk_end(w);  // no further leaf
-                        if (FIRST) {
-                            walk_centroid_deposit<A>(P, walk_tet(w));  // (periodic: never outside the tree)
-                            cnt.add_dep(P.m_tet);
-                            if (STATS) { cnt.u[ST_DEGENERATE]++; cnt.u[ST_OVERLAPPED]++; }
-                        }
-                    }
-                }
+                const bool first_pair = fresh;
+                const bool degenerate = first_pair && !(ts.kappa <= 1e4f) && walk_det6(P, walk_tet(w)) == 0.0;
+                bool to_centroid = degenerate;
                 fresh = false;
 #pragma unroll
                 for (int q = 0; q < 4; ++q) res[q] = mk<float>(0.f, 0.f, 0.f);
@@ -644,15 +635,26 @@ __global__ void __launch_bounds__(128, MINB) k_oct_warp(const DepositParams P)
                         dim[a] = hi - lo[a] + 1;
                     }
                     const int64_t ncell = (int64_t)dim[0] * dim[1] * dim[2];
-                    if (!FIRST && (single || !guard)) {
+                    if (single) {
+                        // The whole tetrahedron goes to one cell of this leaf, and the walk ends.  Float32
+                        // rounding can put that cell beside the leaf that the float64 nodes name, or into
+                        // one of two leaves that they name: a cell outside the block (an empty range) is
+                        // never written; at the first leaf the centroid decides, later leaves get nothing
+                        const bool here = ncell == 1 && (dim[0] | dim[1] | dim[2]) == 1;
+                        if (here) {
+                            walk_end(w);
+                            if (FIRST) {
+                                cell_add<A>(P, P.out + ((leaf * (int64_t)bc + (lo[2] - org[2])) * (bc * bc) +
+                                                        (lo[0] - org[0] + bc * (lo[1] - org[1]))),
+                                            P.m_tet);
+                                cnt.add_dep(P.m_tet);
+                                if (STATS) { cnt.u[ST_SINGLE_CELL]++; cnt.u[ST_BBOX_CELLS]++; cnt.u[ST_OVERLAPPED]++; }
+                            }
+                        } else {
+                            to_centroid = first_pair;
+                        }
+                    } else if (!FIRST && !guard) {
                         // the guarded pass: nothing to do for this pair
-                    } else if (single) {
-                        // whole tetrahedron inside one cell of this leaf
-                        cell_add<A>(P, P.out + ((leaf * (int64_t)bc + (lo[2] - org[2])) * (bc * bc) +
-                                                (lo[0] - org[0] + bc * (lo[1] - org[1]))),
-                                    P.m_tet);
-                        cnt.add_dep(P.m_tet);
-                        if (STATS) { cnt.u[ST_SINGLE_CELL]++; cnt.u[ST_BBOX_CELLS]++; cnt.u[ST_OVERLAPPED]++; }
                     } else if (ncell > (int64_t)(1 << 25) || !dims_fit_queue(dim)) {
                         set_error(P.ws, 2, lane);
                     } else if (FIRST && guard) {
@@ -670,6 +672,14 @@ __global__ void __launch_bounds__(128, MINB) k_oct_warp(const DepositParams P)
                         const int C = ts.axis;
                         const bool cut = C == 0 ? lo[0] > ts.lo[0] : (C == 1 ? lo[1] > ts.lo[1] : lo[2] > ts.lo[2]);
                         store_record<PASS>(S, lane, ts, res, lo, dim, org, P.m_tet, P.kappa_max, cut);
+                    }
+                }
+                if (to_centroid) {
+                    walk_end(w);  // no further leaf
+                    if (FIRST) {
+                        walk_centroid_deposit<A>(P, walk_tet(w));  // (periodic: never outside the tree)
+                        cnt.add_dep(P.m_tet);
+                        if (STATS) { cnt.u[degenerate ? ST_DEGENERATE : ST_SINGLE_CELL]++; cnt.u[ST_OVERLAPPED]++; }
                     }
                 }
             }
