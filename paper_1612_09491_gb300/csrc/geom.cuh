@@ -548,6 +548,20 @@ PSE_HD bool tet_setup(P3<T> (&v)[4], TetSetup<T> &s)
     return d6 < 0.0;
 }
 
+// Whether the exact tetrahedron may be degenerate (6V = 0), from the set-up of its float32
+// vertices: kappa and |6V|.  Their rounding moves a vertex by at most d = 1.1e-7 (lmax + unit)
+// cells: unit = 2 (coordinates in the base cell's frame), plus the grid's cells a side if vertices are
+// taken at a periodic image (the scale's own rounding; without images it keeps planes plane).  That
+// changes 6V by d area2 at first order, area2 the sum of the normals' lengths, while |6V| = area2
+// lmax / kappa; so 6V was not 0 where kappa <= 1e4 and lmax >= cbrt(|6V|) > 1e-6 kappa unit, with a factor
+// of 5 to spare after the higher orders.  An exactly flat tetrahedron of a few float32 steps is far
+// below that size, though its kappa may be a few hundred.
+PSE_HD bool may_be_flat(float kappa, float vol6, float unit)
+{
+    const float t = 1e-6f * kappa * unit;
+    return !(kappa <= 1e4f && vol6 > t * t * t);
+}
+
 // Cell classification for the cell with corner c (base-cell frame, integers).
 enum { CELL_OUTSIDE = 0, CELL_INSIDE = 1, CELL_PARTIAL = 2 };
 

@@ -602,10 +602,11 @@ __global__ void __launch_bounds__(128, MINB) k_oct_warp(const DepositParams P)
                 TetSetup<float> ts;
                 const bool swapped = tet_setup<float>(v, ts);
                 const bool guard = !(ts.kappa <= P.kappa_max);
-                // Exactly degenerate tetrahedra go to the cell of their centroid, once.  Up to kappa
-                // = 1e4 a tetrahedron cannot be degenerate: its rounded volume is right to 1%
+                // Exactly degenerate tetrahedra go to the cell of their centroid, once
                 const bool first_pair = fresh;
-                const bool degenerate = first_pair && !(ts.kappa <= 1e4f) && walk_det6(P, walk_tet(w)) == 0.0;
+                const float unit = w.shifts != 0 ? (float)(2 + ((int64_t)P.bc << level)) : 2.f;
+                const bool degenerate =
+                    first_pair && may_be_flat(ts.kappa, (float)ts.vol6, unit) && walk_det6(P, walk_tet(w)) == 0.0;
                 bool to_centroid = degenerate;
                 fresh = false;
 #pragma unroll

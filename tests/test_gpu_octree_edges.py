@@ -91,3 +91,51 @@ def test_single_cell_across_a_leaf_plane(prec, cap):
     # beside the plane: the last cell of the leaf below it, the first one of the leaf above
     assert got[node - 1, 5, 5, bc - 1] + got[node, 5, 5, 0] == pytest.approx(1.0, abs=1e-12)
     assert float(got.sum()) == pytest.approx(1.0, abs=1e-12)
+
+
+# cells a side over a box whose ratio float32 has to round, so that a plane of float32 positions is no
+# plane any more in cells (box 100 with 24 and 192 cells, 75 with 100, 1 with 100 and 384); 1 and 256: exact
+COPLANAR = [(100.0, 24, 0), (100.0, 24, 3), (75.0, 100, 0), (1.0, 100, 0), (1.0, 24, 4), (1.0, 32, 3)]
+
+
+def coplanar_cluster(box, cells, rng, across=False):
+    """Eight particles of an oblique plane, a few to a few dozen float32 steps wide, on a cell plane
+    (across: on the box boundary, half of them in the image on the other side)."""
+    cell = box / cells
+    while True:
+        c = np.float32(cell * (rng.integers(1, cells, 3) + rng.uniform(0.1, 0.9, 3))).astype(np.float64)
+        ax = rng.integers(3)
+        c[ax] = 0.0 if across else np.float64(np.float32(cell * rng.integers(1, cells)))
+        step = np.array([np.spacing(np.float32(v)) for v in c], np.float64)
+        if across:
+            step[:] = np.spacing(np.float32(box * (1 - 1e-6)))
+            c = np.round(c / step) * step
+        w = int(rng.integers(1, 20))
+        a, b = rng.integers(-w, w + 1, 3), rng.integers(-w, w + 1, 3)
+        m, n = rng.integers(-2, 3, 2)
+        d = a * m + b * n
+        p = np.array([c + step * (a * i + b * j + d * k) for k in (0, 1) for j in (0, 1) for i in (0, 1)])
+        p = np.where(p < 0, p + box, p)
+        if np.array_equal(p.astype(np.float32).astype(np.float64), p) and np.linalg.matrix_rank(np.array([a, b])) == 2:
+            return p
+
+
+@pytest.mark.parametrize("across", [False, True])
+@pytest.mark.parametrize("box,bc,level", COPLANAR)
+def test_coplanar_clusters(box, bc, level, across):
+    """Exactly coplanar tetrahedra go whole to their centroid's cell, as in the thread kernel, also
+    where float32 rounding gives them a volume."""
+    rng = np.random.default_rng(7)
+    nn = 1 << level
+    leaves = [(level, x, y, z) for z in range(nn) for y in range(nn) for x in range(nn)]
+    tree = pse.octree_from_leaves(np.array(leaves, np.int32), bc, level, box)
+    big = bc ** 3 * nn ** 3 > 1 << 23
+    for _ in range(4 if big else 25):
+        pos = torch.from_numpy(coplanar_cluster(box, bc * nn, rng, across).astype(np.float32)).cuda()
+        kw = {"box": box, "particle_mass": 0.125, "mass_fixup": False}
+        ref = pse.deposit_octree(pos, 2, tree, schedule=pse.PSE_THREAD_PER_TET, precision=pse.PSE_FP64_PLAIN, **kw)
+        assert float(ref.sum()) == pytest.approx(1.0, abs=1e-12)
+        for prec in WARP:
+            got, st = pse.deposit_octree(pos, 2, tree, precision=prec, stats=True, **kw)
+            assert st["degenerate_tets"] == 48
+            assert float((got - ref).abs().max()) <= 1e-12
