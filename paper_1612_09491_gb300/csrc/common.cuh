@@ -38,11 +38,13 @@ __device__ __forceinline__ int safe_floor(double x)
     return (x > -1073741824.0 && x < 1073741824.0) ? (int)floor(x) : kBadCoord;
 }
 
-// A tetrahedron is processed only if its base cell and bounding box are sane.
+// A tetrahedron is processed only if its base cell, bounding box and volume are sane.  A NaN
+// coordinate drops out of the bounding box's minima and maxima but not of the volume (its bits are
+// compared: no float64 instruction).
 template <class T>
 __device__ __forceinline__ bool tet_ok(const int (&base)[3], const TetSetup<T> &ts)
 {
-    bool ok = true;
+    bool ok = (__double2hiint(ts.vol6) & 0x7fffffff) < 0x7ff00000;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         ok = ok && base[a] != kBadCoord && ts.dim[a] >= 1 && ts.dim[a] <= (1 << 24) &&
