@@ -114,10 +114,12 @@ std::vector<GraphEntry> g_graphs;       // most recently used last
 constexpr size_t kMaxGraphs = 16;
 cudaStream_t g_capture_stream[64] = {};
 
-std::string graph_key(const pse::DepositParams &p, int64_t cells, bool accumulate, bool renorm, int bps)
+// everything that the launch sequence depends on: the kernels' parameters, and what selects the kernels
+std::string graph_key(const pse::DepositParams &p, const pse_deposit_opts &o, bool thread_fp64, int64_t cells,
+                      bool renorm, int bps)
 {
     std::string k(reinterpret_cast<const char *>(&p), sizeof(p));
-    const int64_t extra[4] = {cells, accumulate ? 1 : 0, renorm ? 1 : 0, bps};
+    const int64_t extra[7] = {cells, o.accumulate ? 1 : 0, renorm ? 1 : 0, bps, o.precision, o.schedule, thread_fp64 ? 1 : 0};
     k.append(reinterpret_cast<const char *>(extra), sizeof(extra));
     return k;
 }
@@ -343,6 +345,7 @@ int run_deposit(pse::DepositParams &p, const pse_deposit_opts &o, int64_t cells,
     const bool comp = o.precision == PSE_FP32_COMPENSATED;
     p.comp = comp ? 1 : 0;
     const int bps = (tu && tu->blocks_per_sm > 0) ? tu->blocks_per_sm : kDefaultBlocksPerSm;
+    const bool thread_fp64 = tu && tu->thread_fp64;
     set_items(p, cells);
 
     // the kernels of one deposit pass over the tetrahedra of q, on stream s
@@ -356,7 +359,7 @@ int run_deposit(pse::DepositParams &p, const pse_deposit_opts &o, int64_t cells,
         } else {
             // float64: the column clip, unless the call counts cells (the thread kernel's counters
             // are per cell) or asks for the thread kernel
-            if (o.precision == PSE_FP64_PLAIN && !stats && !(tu && tu->thread_fp64)) e = pse::launch_warp_plain(q, s);
+            if (o.precision == PSE_FP64_PLAIN && !stats && !thread_fp64) e = pse::launch_warp_plain(q, s);
             else if (o.schedule == PSE_THREAD_PER_TET) e = pse::launch_thread_per_tet(q, o.precision == PSE_FP64_PLAIN, stats, s);
             else if (o.schedule == PSE_WARP_PER_TET) e = pse::launch_warp_per_tet(q, stats, s);
             else if (binned) e = pse::launch_binned(q, stats, bps, s);
@@ -410,7 +413,7 @@ int run_deposit(pse::DepositParams &p, const pse_deposit_opts &o, int64_t cells,
         e = cudaGetDevice(&dev);
         if (e != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
         if (dev < 0 || dev >= 64) return fail(PSE_ERR_UNSUPPORTED, "device index beyond the supported range");
-        const std::string key = graph_key(p, cells, o.accumulate != 0, renorm, bps);
+        const std::string key = graph_key(p, o, thread_fp64, cells, renorm, bps);
         std::lock_guard<std::mutex> lk(g_graph_mu);
         cudaGraphExec_t exec = nullptr;
         for (size_t i = 0; i < g_graphs.size(); ++i)
