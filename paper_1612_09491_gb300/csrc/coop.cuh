@@ -23,7 +23,7 @@ namespace {
 // Split work item `item` of the binned schedule: chunk [first, first + len) of the
 // bounding-box cells of one queued tetrahedron, set up by lane 0 as record 0.  Returns
 // the lane's pair count (len on lane 0, else 0).
-template <bool STATS, int PASS>
+template <bool STATS, Acc A, int PASS>
 __device__ __forceinline__ int chunk_setup(const DepositParams &P, WarpSmem *S, int lane, int64_t item, int64_t q,
                                            int &skip, Counters &cnt)
 {
@@ -62,6 +62,15 @@ __device__ __forceinline__ int chunk_setup(const DepositParams &P, WarpSmem *S, 
     // each pass takes the pieces of its own side of the guard
     const bool guard = !(ts.kappa <= P.kappa_max);
     if (guard != (PASS == kPassGuard)) return 0;
+    int c[3];
+    if (PASS == kPassGuard && flat_guarded(P, ts, res, base, id, c)) {  // once, with the first piece
+        if (first == 0) {
+            if (!deposit_cell<A>(P, c[0], c[1], c[2], m_t) && STATS) cnt.dropped += m_t;
+            cnt.add_dep(m_t);
+            if (STATS) { cnt.u[ST_DEGENERATE]++; cnt.u[ST_OVERLAPPED]++; }
+        }
+        return 0;
+    }
     store_record<PASS>(S, 0, ts, res, ts.lo, ts.dim, base, m_t, P.kappa_max, false);
     return len;
 }
@@ -164,7 +173,7 @@ __global__ void __launch_bounds__(kCoopThreads, MINB) k_warp_coop(const DepositP
             int64_t tid = 0;
             bool to_list = false;
             if (is_chunk) {
-                npairs = chunk_setup<STATS, PASS>(P, S, lane, (int64_t)item, q, skip, cnt);
+                npairs = chunk_setup<STATS, A, PASS>(P, S, lane, (int64_t)item, q, skip, cnt);
                 __syncwarp();
             } else if (unit >= 0) {
                 P3<float> v[4];
@@ -232,13 +241,19 @@ __global__ void __launch_bounds__(kCoopThreads, MINB) k_warp_coop(const DepositP
                 } else {
                     // guarded: column runs, clipped in float64 from the exact vertices
                     // (the float32 vertices plus their rounding residuals)
-                    npairs = (int)run_count(ts.dim, ts.axis);
                     P3<float> res[4], v2[4];
-                    int b2[3];
+                    int b2[3], c[3];
                     if (P.src == SRC_TETS) explicit_tet<float>(P, unit, v2, b2, res);
                     else lattice_tet<float>(P, ci, cj, ck, s, v2, b2, res);
                     if (swapped) swap12(res);
-                    store_record<PASS>(S, lane, ts, res, ts.lo, ts.dim, base, m_t, P.kappa_max, false);
+                    if (flat_guarded(P, ts, res, base, tid, c)) {
+                        if (!deposit_cell<A>(P, c[0], c[1], c[2], m_t) && STATS) cnt.dropped += m_t;
+                        cnt.add_dep(m_t);
+                        if (STATS) { cnt.u[ST_DEGENERATE]++; cnt.u[ST_OVERLAPPED]++; }
+                    } else {
+                        npairs = (int)run_count(ts.dim, ts.axis);
+                        store_record<PASS>(S, lane, ts, res, ts.lo, ts.dim, base, m_t, P.kappa_max, false);
+                    }
                 }
             }
             if (FIRST && !BINNED) list_guarded(P, to_list, tid, lane);

@@ -77,6 +77,13 @@ __global__ void __launch_bounds__(128) k_thread_per_tet(const DepositParams P)
             if (STATS) { cnt.u[ST_SINGLE_CELL]++; cnt.u[ST_OVERLAPPED]++; }
             continue;
         }
+        int c[3];
+        if (flat_cell(P, ts, t, c)) {
+            if (!deposit_cell(P, c[0], c[1], c[2], m_t) && STATS) cnt.dropped += m_t;
+            cnt.add_dep(m_t);
+            if (STATS) { cnt.u[ST_DEGENERATE]++; cnt.u[ST_OVERLAPPED]++; }
+            continue;
+        }
         // FP32 guard: ill-conditioned tetrahedra are clipped in float64 from their exact vertices
         const bool g64 = (sizeof(T) == 4) && !(ts.kappa <= P.kappa_max);
         double rho = 6.0 * m_t / ts.vol6;
@@ -238,6 +245,8 @@ __global__ void __launch_bounds__(kCoopThreads, 2) k_warp_plain(const DepositPar
                 int c[3];
                 centroid_cell(v, c);
                 deposit_cell<Acc::F64>(P, base[0] + c[0], base[1] + c[1], base[2] + c[2], m_t);
+            } else if (int c[3]; ncell > 1 && flat_cell(P, ts, P.src == SRC_TETS ? u : 6 * u + s, c)) {
+                deposit_cell<Acc::F64>(P, c[0], c[1], c[2], m_t);
             } else if (ncell == 1) {
                 deposit_cell<Acc::F64>(P, base[0] + ts.lo[0], base[1] + ts.lo[1], base[2] + ts.lo[2], m_t);
             } else if (ncell > (int64_t)(1 << 25) || !dims_fit_queue(ts.dim)) {
@@ -341,6 +350,16 @@ __global__ void __launch_bounds__(kCoopThreads, 2) k_warp_per_tet(const DepositP
                         cnt.u[ts.vol6 == 0.0 ? ST_DEGENERATE : ST_SINGLE_CELL]++;
                         cnt.u[ST_OVERLAPPED]++;
                         if (ts.vol6 != 0.0) { cnt.u[ST_BBOX_CELLS]++; cnt.u[ST_BIN0]++; }
+                    }
+                } else if (int c[3]; !(ts.kappa <= P.kappa_max) && flat_guarded(P, ts, res, base, (int64_t)t, c)) {
+                    if (!deposit_cell(P, c[0], c[1], c[2], m_t) && STATS) cnt.dropped += m_t;
+                    cnt.add_tgt(P, m_t);
+                    cnt.add_dep(m_t);
+                    if (STATS) {
+                        cnt.u[ST_DEGENERATE]++;
+                        cnt.u[ST_OVERLAPPED]++;
+                        cnt.u[ST_BBOX_CELLS] += ncell;
+                        cnt.u[ST_BIN0 + size_bin(ncell)]++;
                     }
                 } else if (ncell > (int64_t)(1 << 25) || !dims_fit_queue(ts.dim)) {
                     set_error(P.ws, 2, (int)(t & 0x7fffffff));
