@@ -136,35 +136,40 @@ __global__ void __launch_bounds__(128) k_thread_per_tet(const DepositParams P)
 // ---------------------------------------------------------------------------
 // every step in float64, by the warp-cooperative column clip
 // ---------------------------------------------------------------------------
-// Cell by cell for a tetrahedron that the run queue cannot hold (2^25 cells and more): its own
-// thread, as k_thread_per_tet does.
-__device__ __noinline__ void plain_cells(const DepositParams &P, TetSetup<double> ts, int bx, int by, int bz, double rho)
+// Cell by cell for a tetrahedron that the run queue cannot hold (more than 2^25 cells, or 2^19 and more
+// on a side), record t: its cells dealt to the lanes in turn.
+__device__ __noinline__ void plain_cells(const DepositParams &P, WarpSmem *S, int t, int lane)
 {
-    for (int iz = 0; iz < ts.dim[2]; ++iz)
-        for (int iy = 0; iy < ts.dim[1]; ++iy)
-            for (int ix = 0; ix < ts.dim[0]; ++ix) {
-                const int cx = ts.lo[0] + ix, cy = ts.lo[1] + iy, cz = ts.lo[2] + iz;
-                const int cls = classify_cell<double>(ts.n, ts.e, ts.pos, ts.neg, (double)cx, (double)cy, (double)cz);
-                double vol = cls == CELL_INSIDE ? 1.0 : 0.0;
-                if (cls == CELL_PARTIAL) {
-                    P3<double> p[4];
+    const GuardSmem *G = guard_smem(S);
+    P3<double> v[4];
 #pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        p[q] = mk<double>(ts.v[q].x - cx, ts.v[q].y - cy, ts.v[q].z - cz);
-                    double err;
-                    vol = overlap_volume_ax<double>(p, ts.n, ts.axis, ts.lx, ts.ly, err);
-                }
-                if (vol > 0.0) deposit_cell<Acc::F64>(P, bx + cx, by + cy, bz + cz, rho * vol);
-            }
-}
-__device__ __noinline__ void plain_large(const DepositParams &P, double x0, double y0, double z0, double x1, double y1,
-                                         double z1, double x2, double y2, double z2, double x3, double y3, double z3,
-                                         int bx, int by, int bz, double m_t)
-{
-    P3<double> v[4] = {mk<double>(x0, y0, z0), mk<double>(x1, y1, z1), mk<double>(x2, y2, z2), mk<double>(x3, y3, z3)};
+    for (int q = 0; q < 4; ++q) v[q] = mk<double>(G->v[3 * q][t], G->v[3 * q + 1][t], G->v[3 * q + 2][t]);
     TetSetup<double> ts;
     tet_setup<double>(v, ts);
-    plain_cells(P, ts, bx, by, bz, 6.0 * m_t / ts.vol6);
+    const double rho = G->rho[t];
+    const int bx = S->base[0][t], by = S->base[1][t], bz = S->base[2][t];
+    // cell number lane, then 32 on: each coordinate moves by less than its range, with one carry
+    const int dx = ts.dim[0], dy = ts.dim[1];
+    const int sx = 32 % dx, sy = 32 / dx % dy, sz = 32 / dx / dy;
+    int ix = lane % dx, iy = lane / dx % dy, iz = lane / dx / dy;
+    while (iz < ts.dim[2]) {
+        const int cx = ts.lo[0] + ix, cy = ts.lo[1] + iy, cz = ts.lo[2] + iz;
+        const int cls = classify_cell<double>(ts.n, ts.e, ts.pos, ts.neg, (double)cx, (double)cy, (double)cz);
+        double vol = cls == CELL_INSIDE ? 1.0 : 0.0;
+        if (cls == CELL_PARTIAL) {
+            P3<double> p[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) p[q] = mk<double>(ts.v[q].x - cx, ts.v[q].y - cy, ts.v[q].z - cz);
+            double err;
+            vol = overlap_volume_ax<double>(p, ts.n, ts.axis, ts.lx, ts.ly, err);
+        }
+        if (vol > 0.0) deposit_cell<Acc::F64>(P, bx + cx, by + cy, bz + cz, rho * vol);
+        ix += sx;
+        if (ix >= dx) { ix -= dx; ++iy; }
+        iy += sy;
+        if (iy >= dy) { iy -= dy; ++iz; }
+        iz += sz;
+    }
 }
 
 // PSE_FP64_PLAIN without statistics: the warp-cooperative schedule with the guarded pass's
@@ -202,6 +207,7 @@ __global__ void __launch_bounds__(kCoopThreads, 2) k_warp_plain(const DepositPar
             have = false;
         }
         int npairs = 0;
+        bool large = false;
         if (have) {
             P3<double> v[4];
             int base[3];
@@ -249,11 +255,9 @@ __global__ void __launch_bounds__(kCoopThreads, 2) k_warp_plain(const DepositPar
                 deposit_cell<Acc::F64>(P, c[0], c[1], c[2], m_t);
             } else if (ncell == 1) {
                 deposit_cell<Acc::F64>(P, base[0] + ts.lo[0], base[1] + ts.lo[1], base[2] + ts.lo[2], m_t);
-            } else if (ncell > (int64_t)(1 << 25) || !dims_fit_queue(ts.dim)) {
-                plain_large(P, v[0].x, v[0].y, v[0].z, v[1].x, v[1].y, v[1].z, v[2].x, v[2].y, v[2].z, v[3].x, v[3].y,
-                            v[3].z, base[0], base[1], base[2], m_t);
             } else {
-                npairs = (int)run_count(ts.dim, ts.axis);
+                large = ncell > (int64_t)(1 << 25) || !dims_fit_queue(ts.dim);
+                npairs = large ? 0 : (int)run_count(ts.dim, ts.axis);
                 const float l1 = 1.f + (float)max(ts.dim[0], max(ts.dim[1], ts.dim[2])), margin = 1e-6f * l1 * l1 * l1;
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
@@ -282,6 +286,10 @@ __global__ void __launch_bounds__(kCoopThreads, 2) k_warp_plain(const DepositPar
                 G->rho[lane] = 6.0 * m_t / vol6;
                 G->tol[lane] = f64_tolerance((double)(ts.dim[0] + ts.dim[1] + ts.dim[2]));
             }
+        }
+        for (unsigned left = __ballot_sync(kFull, large); left != 0u; left &= left - 1u) {
+            __syncwarp();  // the records are written
+            plain_cells(P, S, __ffs((int)left) - 1, lane);
         }
         coop_runs<false, false, Acc::F64, double, true>(P, S, lane, npairs, 0, cnt);
         __syncwarp();
