@@ -472,8 +472,8 @@ PSE_HD T level_volume(T c0, T c1, T s0, T s1, T colmin, T colmax, T msum)
 // operations: 1 in 2.5 of the generic stages above.
 //  * Comparisons, minima and clamps read the numbers' bits (ordered as integers) instead of
 //    the float64 pipe.
-//  * The reciprocal of an edge's extent starts from the float32 one and takes one third-order
-//    step, r (1 + e + e^2) with e = 1 - x r (the error falls from 1e-7 to below rounding).
+//  * The reciprocal of an edge's extent starts from the float32 one and takes one step of
+//    Chebyshev's iteration, r (1 + e + e^2) with e = 1 - x r (the error falls from 1e-7 to below rounding).
 //  * All integrals of a polygon come from four moments, Σ C, Σ C (x_a + x_b), Σ C (y_a + y_b) and
 //    Σ C (z_a + z_b), with C the cross product of an edge's ends about one of the polygon's own
 //    vertices (in the cell, so nothing cancels).
@@ -534,7 +534,9 @@ PSE_HD double f64_widen(float x)
 #endif
 }
 
-// 1 / x (0 for an x beyond 2^-100 .. 2^100: an edge that does not cross anything)
+// 1 / x (0 for an x beyond 2^-100 .. 2^100: an edge that does not cross anything), within an ulp: the float32
+// reciprocal of x cut to float32 (error e below 2^-21), then one step of Chebyshev's iteration for 1 / x
+// (Altman's hyperpower method of order three), which leaves e^3
 PSE_HD double f64_rcp(double x)
 {
 #ifdef __CUDA_ARCH__
