@@ -181,8 +181,8 @@ void set_items(pse::DepositParams &p, int64_t cells)
     const int64_t tets = p.n_units * nsub, waves = (tets + 32 * kWarps - 1) / (32 * kWarps);
     p.group = tets > 0 ? (int)((tets + kWarps * waves - 1) / (kWarps * waves)) : 32;
     const int64_t groups = (p.n_units + p.group - 1) / p.group;
-    p.subs = (p.leaves && groups >= 4 * kWarps) ? 6 : 1;
-    p.n_items = groups * (nsub / (p.leaves ? p.subs : 1));
+    p.subs = (p.leaves && nsub == 6 && groups >= 4 * kWarps) ? 6 : 1;
+    p.n_items = groups * (nsub / p.subs);
     if (p.slab) return;  // a slab keeps the whole lattice's choice
     p.pace = (p.src != pse::SRC_TETS && (double)cells <= kPaceCells * (double)p.nc[0] * (double)p.nc[1] * (double)p.nc[2])
                  ? 1 : 0;
