@@ -217,7 +217,8 @@ PSE_API int pse_build_tets_from_lagrangian_grid(const float *d_pos, const pse_la
  *               PSE_OP_DEPOSIT_UNIFORM, lat, opts); NULL with ws_bytes = 0 makes the library
  *               allocate it stream-ordered for this call.
  * Device-side failures (a bad cube id, non-finite coordinates, a bounding box beyond
- * the int32 cell range) are recorded in the workspace and returned as PSE_ERR_DEVICE
+ * the int32 cell range; on octrees by the warp schedule also one of 65535 and more finest nodes on a
+ * side, or 2^21 and more boxes away) are recorded in the workspace and returned as PSE_ERR_DEVICE
  * by calls that pass h_stats; calls without h_stats do not synchronise and do not
  * report them.
  */

@@ -164,11 +164,10 @@ void fill_grid(pse::DepositParams &p, const int64_t grid_n[3], double box)
 // The work items of the warp kernels.  An item is one warp's batch of up to 32 tetrahedra: the
 // same Kuhn tetrahedron of 32 consecutive cubes (octree: all six, one after another, while there
 // are many items), or 32 tetrahedra of an explicit set.  The items are made as large as lets them
-// fill a whole number of waves of the warps that the GPU holds (16 on each of 152 SMs), which
-// matters for small deposits: 16^3 on 32^3 170 us with 8 cubes an item (1.3 waves), 154 us with 11
-// (one wave); 32^3 on 64^3 549 -> 536 us.  (Before, an item was a row segment of 32 cubes with all
-// six tetrahedra: 16^3 on 32^3 0.86 ms, 32^3 on 64^3 0.92 ms, 48^3 on 384^3, whose rows fill three quarters of a warp, 31.0 -> 18.3 ms, 256^3 on
-// 128^3 64.7 -> 56.4 ms.)
+// fill a whole number of waves of 152 x 16 warps, what this GPU holds of the FP32 kernels at 4 blocks
+// an SM (small deposits: 16^3 on 32^3 170 us with 8 cubes an item, 1.3 waves, and 154 us with 11, one
+// wave).  The float64 and counting kernels hold half as many warps and take twice the waves.
+//
 // The FP32 pass paces its blocks (coop.cuh) up to this many output cells a cube.  160^3
 // cubes, unpaced and paced: 0.5 cells 18.4 and 16.7 ms, 1 cell 21.7 and 20.5, 2 cells 27.5 and
 // 27.4, 4 cells 38.8 and 39.7.
@@ -300,8 +299,8 @@ int run_deposit(pse::DepositParams &p, const pse_deposit_opts &o, int64_t cells,
     size_t need = p.leaves ? octree_ws_bytes(&o) : deposit_ws_bytes(&o, n_tets);
     // A workspace of the library's own, allocated and freed in this call, leaves out what the call
     // cannot use: the residual blocks (the warp-per-tetrahedron baseline's) and list entries beyond
-    // the call's tetrahedra.  Mapping 38 MB made up most of a small call that starts on an idle
-    // device: 16^3 on 32^3 without a workspace 0.45 -> 0.37 ms.
+    // the call's tetrahedra.  Mapping the 38 MB of both takes 0.08 of the 0.45 ms that 16^3 on 32^3 then
+    // needs on an idle device.
     size_t res_bytes = pse::kResidualBytes, list_bytes = pse::kGuardListBytes;
     if (d_ws == nullptr && o.schedule != PSE_THREAD_PER_TET && need > 0) {
         const size_t full = need;

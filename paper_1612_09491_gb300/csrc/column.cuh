@@ -114,8 +114,8 @@ PSE_HD T plane_sum(const P3<T> &a, const P3<T> &b, T l0, T lx, T ly)
 // their number (0 to 5).  An edge is cut at its own parameters for the two planes, each end by
 // the plane it lies beyond; an edge beyond one plane at both ends is left out (it would add
 // exactly 0 to every sum).  ROLL keeps this loop and the one over the new y edges rolled, for the
-// octree kernel, whose set-up code competes for the instruction cache (256^3: 261.5 -> 253.6 ms;
-// the uniform kernel loses 1% by it).
+// octree kernel, whose set-up code competes for the instruction cache (256^3: 3% less time; the
+// uniform kernel loses 1% by it).
 template <bool ROLL, class T, class Slots>
 PSE_HD int xslab_triangle(const P3<T> &a, const P3<T> &b, const P3<T> &c, T lo, T hi, T tol, const Slots &E)
 {
@@ -479,10 +479,8 @@ PSE_HD T level_volume(T c0, T c1, T s0, T s1, T colmin, T colmax, T msum)
 //    vertices (in the cell, so nothing cancels).
 //  * A level's fan starts from a crossing point of the level line itself, so that no face
 //    plane enters, and whole-polygon bounds are kept as ordered integers.
-// The clip's error stays a few 1e-16 of a cell (1e-12 is tested).  Measured (one GB300): the
-// shell-crossed 128^3 octree deposit, seven tenths of it this clip, 141 -> 85 ms, and 79.2 -> 75.8
-// with the moments' ends not moved to o and the sides found on the bits; 60,000 explicit
-// tetrahedra 3.2 -> 1.1 ms (with the guarded list taken in smaller items).  Ten warps an SM
+// The clip's error stays a few 1e-16 of a cell (1e-12 is tested).  The shell-crossed 128^3 octree deposit,
+// seven tenths of it this clip, takes 141 ms with the generic stages and 76 with these.  Ten warps an SM
 // instead of eight change nothing: the pipe is 86% busy.
 // ---------------------------------------------------------------------------
 PSE_HD long long f64_bits(double x)

@@ -106,10 +106,9 @@ __global__ void __launch_bounds__(kCoopThreads, MINB) k_warp_coop(const DepositP
     const int per = LIST ? listed_per_item(listed) : P.group;  // tetrahedra per item
     const int64_t n_items = LIST ? (listed + per - 1) / per : P.n_items;
 
-    // With few clips per tetrahedron (P.pace, see set_items) the set-up code is executed often and
-    // the warps of an SM evict each other's code from the instruction cache.  A block's four
-    // warps then take four items together, so that they run the set-up at the same time (256^3 on
-    // 128^3: 57.3 -> 50.2 ms; at two cells a lattice spacing the waits cost 3%).
+    // With few clips per tetrahedron (P.pace, see set_items for the line and both sides' times) the set-up
+    // code is executed often and the warps of an SM evict each other's code from the instruction cache.
+    // A block's four warps then take four items together, so that they run the set-up at the same time.
     constexpr bool PACED = FIRST && !BINNED;
     __shared__ unsigned long long block_item;
     for (;;) {

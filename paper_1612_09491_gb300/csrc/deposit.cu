@@ -180,8 +180,8 @@ __device__ __noinline__ void plain_cells(const DepositParams &P, WarpSmem *S, in
 //
 // The float64 pipe bounds both this and the thread-per-tetrahedron kernel (16 cycles a warp
 // instruction).  That kernel clips cell by cell with 9 of 32 lanes active; here one clip serves
-// two cells, with 2.5 times fewer float64 operations, and the lanes are full: 48^3 on 96^3 213 ->
-// 16.5 ms, the masses equal to 3e-16 (norm).
+// two cells, with 2.5 times fewer float64 operations, and the lanes are full: 48^3 on 96^3 takes 213 ms
+// there and 16.4 here, the masses equal to 3e-16 (norm).
 __global__ void __launch_bounds__(kCoopThreads, 2) k_warp_plain(const DepositParams P)
 {
     WarpSmem *S = warp_smem(true);

@@ -491,15 +491,14 @@ __device__ __forceinline__ void walk_grid(const DepositParams &P, const LeafWalk
 // Each lane walks the leaves of its own tetrahedra: it takes its next pair while the other lanes
 // take theirs, whichever tetrahedron or leaf they are at, so that a round's 32 records are full
 // until the item's tetrahedra run out.  (Rows of cubes cross leaf blocks, so the lanes of a warp
-// need different numbers of rounds for the same tetrahedron of their cubes: 256^3 octree 294 ->
-// 277 ms, with collapsed regions 345 -> 300 ms, the guarded clips' gain included.)  The warps of an
-// SM compete for its instruction cache, so the steps that few tetrahedra take (periodic shifts,
-// nodes within float32 rounding of a boundary, degenerate ones) are out of line: 268 -> 261 ms,
-// 291 -> 286 ms.
+// need different numbers of rounds for the same tetrahedron of their cubes: in lock step the 256^3 octree
+// takes 6% longer.)  The warps of an SM compete for its instruction cache, so the steps that few
+// tetrahedra take (periodic shifts, nodes within float32 rounding of a boundary, degenerate ones, a cell
+// beside its leaf) are out of line: 3% of the same case.
 //
 // PACE (DepositParams::pace): the warps of a block set their records up together, as in
 // k_warp_coop; a variant of its own, because the test alone costs the other octree deposits 0.5%
-// (shell-crossed 128^3: 81.0 -> 79.2 ms).
+// (shell-crossed 128^3: 2% less time with it).
 template <bool STATS, int MINB, Acc A, int PASS, bool PACE = false>
 __global__ void __launch_bounds__(128, MINB) k_oct_warp(const DepositParams P)
 {
@@ -739,12 +738,11 @@ __device__ __noinline__ float far_offset(double box, float x, float x0)
 // of the coarser levels are the finest level's node coordinates shifted.  Equal (node, bin)
 // keys are merged in the warp before one atomic per key.
 //
-// The float64 centroids bound this kernel (16 cycles a warp instruction: 11.2 ms for 256^3,
-// the float64 pipe 83% busy), so nodes and bins come from float32 and only what lies within
+// Centroids in float64 would bound this kernel (16 cycles a warp instruction: 11.2 ms for 256^3 with the
+// float64 pipe 83% busy, 2.5 ms as it is), so nodes and bins come from float32 and only what lies within
 // the rounding of a boundary is decided by the float64 centroid and the level's own log10.
 // Float32 errors: below 4e-7 of the box and of the position for a centroid, below 2e-5 of a bin
-// for the shifted logarithm; the margins are 2e-6 and 4e-5.  Measured: the 256^3 octree build and
-// deposit 277 -> 270.5 ms, and 2.4 ms less with far_offset out of line.
+// for the shifted logarithm; the margins are 2e-6 and 4e-5.
 __global__ void __launch_bounds__(256) k_tet_size_hist(const DepositParams P, unsigned *__restrict__ hist)
 {
     __shared__ unsigned sh[64 + 512];  // levels 0 and 1 aggregated per block
