@@ -229,7 +229,10 @@ __global__ void __launch_bounds__(128) k_oct_thread(const DepositParams P)
         fine_range(P, x, k, f0, f1);
         int64_t cursor = 0;
         LeafHit hit;
+        bool first = true;
         while (next_leaf(P, f0, f1, cursor, hit)) {
+            const bool first_pair = first;
+            first = false;
             P3<T> v[4];
             P3<float> res[4];
             int base[3];
@@ -249,46 +252,50 @@ __global__ void __launch_bounds__(128) k_oct_thread(const DepositParams P)
                 hi[a] = ts.lo[a] + ts.dim[a] - 1 < org[a] + (int)bc - 1 ? ts.lo[a] + ts.dim[a] - 1 : org[a] + (int)bc - 1;
             }
             const bool single = ts.dim[0] == 1 && ts.dim[1] == 1 && ts.dim[2] == 1;
-            const bool g64 = (sizeof(T) == 4) && !(ts.kappa <= P.kappa_max) && !single;
+            const bool g64 = (sizeof(T) == 4) && !(ts.kappa <= P.kappa_max);
             double rho = 6.0 * m_t / ts.vol6;
             if constexpr (sizeof(T) == 4) {
                 if (g64) rho = 6.0 * m_t / exact_vol6(ts.v, res, ts.vol6);
             }
             double* blk = P.out + (int64_t)hit.leaf * bc * bc * bc;
+            if (single) {  // whole, to one cell, once: as in k_oct_warp
+                const bool here = lo[0] == hi[0] && lo[1] == hi[1] && lo[2] == hi[2];
+                if (!here && !first_pair) continue;
+                if (here) cell_add(P, blk + (lo[0] - org[0]) + bc * ((lo[1] - org[1]) + bc * (lo[2] - org[2])), m_t);
+                else add_mass(P, cen, m_t, cnt, STATS);
+                cnt.add_dep(m_t);
+                if (STATS) { cnt.u[ST_BBOX_CELLS]++; cnt.u[ST_SINGLE_CELL]++; cnt.u[ST_OVERLAPPED]++; }
+                break;
+            }
             for (int cz = lo[2]; cz <= hi[2]; ++cz)
                 for (int cy = lo[1]; cy <= hi[1]; ++cy)
                     for (int cx = lo[0]; cx <= hi[0]; ++cx) {
                         if (STATS) cnt.u[ST_BBOX_CELLS]++;
                         double vol = 0.0;
-                        if (single) {
-                            vol = ts.vol6 / 6.0;
-                            if (STATS) { cnt.u[ST_SINGLE_CELL]++; cnt.u[ST_OVERLAPPED]++; }
-                        } else {
-                            const int cls = classify_cell<T>(ts.n, ts.e, ts.pos, ts.neg, (T)cx, (T)cy, (T)cz);
-                            if (cls == CELL_INSIDE) {
-                                vol = 1.0;
-                                if (STATS) cnt.u[ST_INSIDE_CELLS]++;
-                            } else if (cls == CELL_PARTIAL) {
-                                P3<T> p[4];
+                        const int cls = classify_cell<T>(ts.n, ts.e, ts.pos, ts.neg, (T)cx, (T)cy, (T)cz);
+                        if (cls == CELL_INSIDE) {
+                            vol = 1.0;
+                            if (STATS) cnt.u[ST_INSIDE_CELLS]++;
+                        } else if (cls == CELL_PARTIAL) {
+                            P3<T> p[4];
 #pragma unroll
-                                for (int q = 0; q < 4; ++q)
-                                    p[q] = mk<T>(ts.v[q].x - (T)cx, ts.v[q].y - (T)cy, ts.v[q].z - (T)cz);
-                                if constexpr (sizeof(T) == 4) {
-                                    if (g64) {
-                                        P3<double> pd[4];
-                                        exact_vertices(ts.v, res, cx, cy, cz, pd);
-                                        vol = overlap_volume_fp64(pd);
-                                        if (STATS) cnt.u[ST_FP64_REDOS]++;
-                                    } else {
-                                        T err;
-                                        vol = (double)overlap_volume_ax<T>(p, ts.n, ts.axis, ts.lx, ts.ly, err);
-                                    }
+                            for (int q = 0; q < 4; ++q)
+                                p[q] = mk<T>(ts.v[q].x - (T)cx, ts.v[q].y - (T)cy, ts.v[q].z - (T)cz);
+                            if constexpr (sizeof(T) == 4) {
+                                if (g64) {
+                                    P3<double> pd[4];
+                                    exact_vertices(ts.v, res, cx, cy, cz, pd);
+                                    vol = overlap_volume_fp64(pd);
+                                    if (STATS) cnt.u[ST_FP64_REDOS]++;
                                 } else {
                                     T err;
                                     vol = (double)overlap_volume_ax<T>(p, ts.n, ts.axis, ts.lx, ts.ly, err);
                                 }
-                                if (STATS) cnt.u[ST_PARTIAL_CLIPS]++;
+                            } else {
+                                T err;
+                                vol = (double)overlap_volume_ax<T>(p, ts.n, ts.axis, ts.lx, ts.ly, err);
                             }
+                            if (STATS) cnt.u[ST_PARTIAL_CLIPS]++;
                         }
                         if (vol > 0.0) {
                             if (STATS) cnt.u[ST_OVERLAPPED]++;

@@ -15,6 +15,9 @@ import paper_1612_09491_gb300 as pse  # noqa: E402
 pytestmark = pytest.mark.gpu
 
 WARP = [pse.PSE_FP32_FP64ACC, pse.PSE_FP32_COMPENSATED]
+# (precision, schedule, guard_list_cap)
+PATHS = [(p, pse.PSE_WARP_COOPERATIVE, cap) for p in WARP for cap in (0, -1)] + \
+    [(p, pse.PSE_THREAD_PER_TET, 0) for p in (pse.PSE_FP32_FP64ACC, pse.PSE_FP64_PLAIN)]
 EIGHTHS = [(1, c & 1, (c >> 1) & 1, c >> 2) for c in range(8)]
 GUARD = 4096  # cells kept around the leaf array to see writes outside it
 
@@ -39,9 +42,8 @@ def deposit(pos, tree, bc, box, **kw):
     return (out.cpu().numpy(), r[1]) if isinstance(r, tuple) else out.cpu().numpy()
 
 
-@pytest.mark.parametrize("cap", [0, -1])
-@pytest.mark.parametrize("prec", WARP)
-def test_single_cell_just_below_the_box(prec, cap):
+@pytest.mark.parametrize("prec,sched,cap", PATHS)
+def test_single_cell_just_below_the_box(prec, sched, cap):
     """z a few 1e-20 below the box: float64 names the last leaf (of the image below), float32
     rounds the cell to the one after it."""
     rng = np.random.default_rng(2)
@@ -50,17 +52,16 @@ def test_single_cell_just_below_the_box(prec, cap):
     pos[:, 2] = -1e-20 * rng.permutation(np.arange(1, 9))
     bc = 4
     tree = pse.octree_from_leaves(np.array(EIGHTHS, np.int32), bc, 1)
-    got, st = deposit(pos, tree, bc, 1.0, precision=prec, stats=True, tuning={"guard_list_cap": cap})
+    got, st = deposit(pos, tree, bc, 1.0, precision=prec, schedule=sched, stats=True, tuning={"guard_list_cap": cap})
     want = np.zeros_like(got)
     want[7, 3, 3, 3] = 1.0
     # (compensated sums hold a cell to 2^-48 of each addend)
     np.testing.assert_allclose(got, want, rtol=0, atol=1e-12)
-    assert st["single_cell_tets"] + st["degenerate_tets"] == 48
+    assert st["single_cell_tets"] + st["degenerate_tets"] == 48 == st["overlapped_cells"]
 
 
-@pytest.mark.parametrize("cap", [0, -1])
-@pytest.mark.parametrize("prec", WARP)
-def test_single_cell_across_a_leaf_plane(prec, cap):
+@pytest.mark.parametrize("prec,sched,cap", PATHS)
+def test_single_cell_across_a_leaf_plane(prec, sched, cap):
     """Cells per box that float32 rounds up: a vertex below a leaf plane lands on it or above, so
     float64 names two leaves and float32 one cell.  Deposited once, beside the plane."""
     box, bc = 33.3, 32
@@ -87,7 +88,7 @@ def test_single_cell_across_a_leaf_plane(prec, cap):
     pos[0, 0] = x
     nodes = [(3, c & 7, (c >> 3) & 7, c >> 6) for c in range(512)]
     tree = pse.octree_from_leaves(np.array(nodes, np.int32), bc, 3, box)
-    got = deposit(pos, tree, bc, box, precision=prec, tuning={"guard_list_cap": cap})
+    got = deposit(pos, tree, bc, box, precision=prec, schedule=sched, tuning={"guard_list_cap": cap})
     # beside the plane: the last cell of the leaf below it, the first one of the leaf above
     assert got[node - 1, 5, 5, bc - 1] + got[node, 5, 5, 0] == pytest.approx(1.0, abs=1e-12)
     assert float(got.sum()) == pytest.approx(1.0, abs=1e-12)
