@@ -39,12 +39,12 @@ __device__ __forceinline__ int safe_floor(double x)
 }
 
 // A tetrahedron is processed only if its base cell, bounding box and volume are sane.  A NaN
-// coordinate drops out of the bounding box's minima and maxima but not of the volume (its bits are
-// compared: no float64 instruction).
+// coordinate drops out of the bounding box's minima and maxima but not of the volume (looked at in
+// float32, as kappa takes it).
 template <class T>
 __device__ __forceinline__ bool tet_ok(const int (&base)[3], const TetSetup<T> &ts)
 {
-    bool ok = (__double2hiint(ts.vol6) & 0x7fffffff) < 0x7ff00000;
+    bool ok = !isnan((float)ts.vol6);
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         ok = ok && base[a] != kBadCoord && ts.dim[a] >= 1 && ts.dim[a] <= (1 << 24) &&
@@ -364,11 +364,34 @@ __device__ __forceinline__ void centroid_cell(const P3<T> (&v)[4], int (&c)[3])
     c[2] = (int)floor(((double)v[0].z + (double)v[1].z + (double)v[2].z + (double)v[3].z) * 0.25);
 }
 
-// 6V of tetrahedron id (unit * 6 + s; of an explicit set its number) is exactly 0 at its float32 positions:
-// float64 in box units, where the products of close positions are exact; the grid units of the set-up
-// round where cells per box is no power of two, and the volume of a flat tetrahedron with them.
-// c: the cell of its centroid (rule of the exactly degenerate ones).  Out of line: few get here.
-__device__ __noinline__ bool exactly_flat(const DepositParams &P, int64_t id, int (&c)[3])
+// Exactly degenerate tetrahedra on uniform grids.  The set-up works in cells, where float32 positions
+// round unless cells per box is a power of two, and with them the volume of a coplanar tetrahedron: dividing by
+// it gives any density.
+//
+// near_flat: whether the volume in cells of a tetrahedron's float64 vertices (of the float32 passes: the float32 ones
+// and their residuals) may be rounding alone.  Their error is at most 6.3e-15 (|coordinates from the box's corner| +
+// extent) cells, 6V's that times the normals' lengths; hardly any tetrahedron is within it.
+__device__ __forceinline__ bool near_flat(const DepositParams &P, double vol6, const int (&dim)[3], const int (&base)[3])
+{
+    const float L = (float)(dim[0] + dim[1] + dim[2]);
+    const float far = (float)(max(abs(base[0]), max(abs(base[1]), abs(base[2]))) + 2) + (float)max(P.g[0], max(P.g[1], P.g[2]));
+    return fabsf((float)vol6) <= 5e-14f * (far + L) * L * L;
+}
+__device__ __forceinline__ bool near_flat(const DepositParams &P, const TetSetup<float> &ts, const P3<float> (&res)[4],
+                                          const int (&base)[3])
+{
+    P3<double> pd[4];
+    exact_vertices(ts.v, res, 0, 0, 0, pd);
+    return near_flat(P, det6(pd), ts.dim, base);
+}
+// (from the float32 vertices alone, for the kernels that set up every tetrahedron and its float64 vertices rarely)
+__device__ __forceinline__ bool near_flat(const DepositParams &P, const TetSetup<float> &ts)
+{
+    return may_be_flat(ts.kappa, (float)ts.vol6, 2.f + (float)max(P.g[0], max(P.g[1], P.g[2])));
+}
+// Such a tetrahedron, id (unit * 6 + s; of an explicit set its number): whether 6V is 0 from its float32 positions, in
+// float64 and box units, where the products of close positions are exact; c: the cell of its centroid.
+__device__ __forceinline__ bool exactly_flat(const DepositParams &P, int64_t id, int (&c)[3])
 {
     float x[4][3];
     unsigned shifts = 0;
@@ -380,32 +403,24 @@ __device__ __noinline__ bool exactly_flat(const DepositParams &P, int64_t id, in
         lattice_positions(P, ci, cj, ck, (int)(id % 6), x);
         shifts = tet_shift_bits(P, x);
     }
-    double u[4][3];
-    for (int q = 0; q < 4; ++q)
-        for (int a = 0; a < 3; ++a) u[q][a] = (double)x[q][a] + (double)shift_of(shifts, q, a) * P.box;
     P3<double> p[4];
-    for (int q = 0; q < 4; ++q) p[q] = mk<double>(u[q][0], u[q][1], u[q][2]);
-    for (int a = 0; a < 3; ++a) c[a] = safe_floor(0.25 * (u[0][a] + u[1][a] + u[2][a] + u[3][a]) * P.scale_d[a]);
+    for (int q = 0; q < 4; ++q)
+        p[q] = mk<double>((double)x[q][0] + (double)shift_of(shifts, q, 0) * P.box,
+                          (double)x[q][1] + (double)shift_of(shifts, q, 1) * P.box,
+                          (double)x[q][2] + (double)shift_of(shifts, q, 2) * P.box);
+    c[0] = safe_floor(0.25 * (p[0].x + p[1].x + p[2].x + p[3].x) * P.scale_d[0]);
+    c[1] = safe_floor(0.25 * (p[0].y + p[1].y + p[2].y + p[3].y) * P.scale_d[1]);
+    c[2] = safe_floor(0.25 * (p[0].z + p[1].z + p[2].z + p[3].z) * P.scale_d[2]);
     return det6(p) == 0.0;
 }
-// exactly_flat, where the set-up's rounding can have made the volume up
-template <class T>
-__device__ __forceinline__ bool flat_cell(const DepositParams &P, const TetSetup<T> &ts, int64_t id, int (&c)[3])
+// If it is flat, m_t goes to that cell.  Returns 0 (not flat, nothing done), 1 (deposited) or 2 (outside an
+// open grid).  Out of line for the hot kernels: few get here.  (The baselines lose 1% and 4% by the call.)
+template <Acc A>
+__device__ __noinline__ int deposit_flat(const DepositParams &P, int64_t id, double m_t)
 {
-    const float unit = P.src == SRC_TETS ? 2.f : 2.f + (float)max(P.g[0], max(P.g[1], P.g[2]));
-    return may_be_flat(ts.kappa, (float)ts.vol6, unit) && exactly_flat(P, id, c);
-}
-// The same for a guarded tetrahedron: the volume of its float64 vertices (float32 ones and residuals) is
-// off by at most 6.3e-15 (|coordinates from the box's corner| + extent) cells x the normals' lengths, so hardly
-// any is looked at (by flat_cell 60,000 explicit tetrahedra took 0.7% longer than without, this way 0.2%).
-__device__ __forceinline__ bool flat_guarded(const DepositParams &P, const TetSetup<float> &ts, const P3<float> (&res)[4],
-                                             const int (&base)[3], int64_t id, int (&c)[3])
-{
-    P3<double> pd[4];
-    exact_vertices(ts.v, res, 0, 0, 0, pd);
-    const float L = (float)(ts.dim[0] + ts.dim[1] + ts.dim[2]);
-    const float far = (float)(max(abs(base[0]), max(abs(base[1]), abs(base[2]))) + 2) + (float)max(P.g[0], max(P.g[1], P.g[2]));
-    return fabsf((float)det6(pd)) <= 5e-14f * (far + L) * L * L && exactly_flat(P, id, c);
+    int c[3];
+    if (!exactly_flat(P, id, c)) return 0;
+    return deposit_cell<A>(P, c[0], c[1], c[2], m_t) ? 1 : 2;
 }
 
 __device__ __forceinline__ int size_bin(int64_t cells)

@@ -62,14 +62,20 @@ __device__ __forceinline__ int chunk_setup(const DepositParams &P, WarpSmem *S, 
     // each pass takes the pieces of its own side of the guard
     const bool guard = !(ts.kappa <= P.kappa_max);
     if (guard != (PASS == kPassGuard)) return 0;
-    int c[3];
-    if (PASS == kPassGuard && flat_guarded(P, ts, res, base, id, c)) {  // once, with the first piece
-        if (first == 0) {
-            if (!deposit_cell<A>(P, c[0], c[1], c[2], m_t) && STATS) cnt.dropped += m_t;
-            cnt.add_dep(m_t);
-            if (STATS) { cnt.u[ST_DEGENERATE]++; cnt.u[ST_OVERLAPPED]++; }
+    if (PASS == kPassGuard && near_flat(P, ts, res, base)) {
+        // an exactly flat one goes to one cell, with its first piece (0 is no mass to the other pieces)
+        const int flat = deposit_flat<A>(P, id, first == 0 ? m_t : 0.0);
+        if (flat != 0) {
+            if (first == 0) {
+                cnt.add_dep(m_t);
+                if (STATS) {
+                    cnt.u[ST_DEGENERATE]++;
+                    cnt.u[ST_OVERLAPPED]++;
+                    if (flat == 2) cnt.dropped += m_t;
+                }
+            }
+            return 0;
         }
-        return 0;
     }
     store_record<PASS>(S, 0, ts, res, ts.lo, ts.dim, base, m_t, P.kappa_max, false);
     return len;
@@ -241,14 +247,18 @@ __global__ void __launch_bounds__(kCoopThreads, MINB) k_warp_coop(const DepositP
                     // guarded: column runs, clipped in float64 from the exact vertices
                     // (the float32 vertices plus their rounding residuals)
                     P3<float> res[4], v2[4];
-                    int b2[3], c[3];
+                    int b2[3];
                     if (P.src == SRC_TETS) explicit_tet<float>(P, unit, v2, b2, res);
                     else lattice_tet<float>(P, ci, cj, ck, s, v2, b2, res);
                     if (swapped) swap12(res);
-                    if (flat_guarded(P, ts, res, base, tid, c)) {
-                        if (!deposit_cell<A>(P, c[0], c[1], c[2], m_t) && STATS) cnt.dropped += m_t;
+                    const int flat = near_flat(P, ts, res, base) ? deposit_flat<A>(P, tid, m_t) : 0;
+                    if (flat != 0) {
                         cnt.add_dep(m_t);
-                        if (STATS) { cnt.u[ST_DEGENERATE]++; cnt.u[ST_OVERLAPPED]++; }
+                        if (STATS) {
+                            cnt.u[ST_DEGENERATE]++;
+                            cnt.u[ST_OVERLAPPED]++;
+                            if (flat == 2) cnt.dropped += m_t;
+                        }
                     } else {
                         npairs = (int)run_count(ts.dim, ts.axis);
                         store_record<PASS>(S, lane, ts, res, ts.lo, ts.dim, base, m_t, P.kappa_max, false);

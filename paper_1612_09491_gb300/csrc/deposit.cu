@@ -77,15 +77,18 @@ __global__ void __launch_bounds__(128) k_thread_per_tet(const DepositParams P)
             if (STATS) { cnt.u[ST_SINGLE_CELL]++; cnt.u[ST_OVERLAPPED]++; }
             continue;
         }
+        // FP32 guard: ill-conditioned tetrahedra are clipped in float64 from their exact vertices
+        const bool g64 = (sizeof(T) == 4) && !(ts.kappa <= P.kappa_max);
+        bool flat;
+        if constexpr (sizeof(T) == 4) flat = g64 && near_flat(P, ts);
+        else flat = near_flat(P, ts.vol6, ts.dim, base);
         int c[3];
-        if (flat_cell(P, ts, t, c)) {
+        if (flat && exactly_flat(P, t, c)) {
             if (!deposit_cell(P, c[0], c[1], c[2], m_t) && STATS) cnt.dropped += m_t;
             cnt.add_dep(m_t);
             if (STATS) { cnt.u[ST_DEGENERATE]++; cnt.u[ST_OVERLAPPED]++; }
             continue;
         }
-        // FP32 guard: ill-conditioned tetrahedra are clipped in float64 from their exact vertices
-        const bool g64 = (sizeof(T) == 4) && !(ts.kappa <= P.kappa_max);
         double rho = 6.0 * m_t / ts.vol6;
         if constexpr (sizeof(T) == 4) {
             if (g64) rho = 6.0 * m_t / exact_vol6(ts.v, res, ts.vol6);
@@ -251,11 +254,10 @@ __global__ void __launch_bounds__(kCoopThreads, 2) k_warp_plain(const DepositPar
                 int c[3];
                 centroid_cell(v, c);
                 deposit_cell<Acc::F64>(P, base[0] + c[0], base[1] + c[1], base[2] + c[2], m_t);
-            } else if (int c[3]; ncell > 1 && flat_cell(P, ts, P.src == SRC_TETS ? u : 6 * u + s, c)) {
-                deposit_cell<Acc::F64>(P, c[0], c[1], c[2], m_t);
             } else if (ncell == 1) {
                 deposit_cell<Acc::F64>(P, base[0] + ts.lo[0], base[1] + ts.lo[1], base[2] + ts.lo[2], m_t);
-            } else {
+            } else if (!near_flat(P, vol6, ts.dim, base) ||
+                       deposit_flat<Acc::F64>(P, P.src == SRC_TETS ? u : 6 * u + s, m_t) == 0) {
                 large = ncell > (int64_t)(1 << 25) || !dims_fit_queue(ts.dim);
                 npairs = large ? 0 : (int)run_count(ts.dim, ts.axis);
                 const float l1 = 1.f + (float)max(ts.dim[0], max(ts.dim[1], ts.dim[2])), margin = 1e-6f * l1 * l1 * l1;
@@ -343,31 +345,27 @@ __global__ void __launch_bounds__(kCoopThreads, 2) k_warp_per_tet(const DepositP
                     cnt.u[ST_INVERTED] += (negative != (P.src != SRC_TETS && kuhn_negative((int)(t % 6)))) ? 1 : 0;
                 }
                 const int64_t ncell = (int64_t)ts.dim[0] * ts.dim[1] * ts.dim[2];
-                if (!tet_ok(base, ts)) {
+                const bool ok_tet = tet_ok(base, ts);
+                int c[3];
+                const bool flat = ok_tet && ts.vol6 != 0.0 && ncell > 1 && !(ts.kappa <= P.kappa_max) && near_flat(P, ts) &&
+                                  exactly_flat(P, (int64_t)t, c);
+                if (!ok_tet) {
                     set_error(P.ws, 4, (int)(t & 0x7fffffff));
-                } else if (ts.vol6 == 0.0 || ncell == 1) {
-                    int c[3];
-                    if (ts.vol6 == 0.0) centroid_cell(ts.v, c);
-                    else { c[0] = ts.lo[0]; c[1] = ts.lo[1]; c[2] = ts.lo[2]; }
-                    if (!deposit_cell(P, base[0] + c[0], base[1] + c[1], base[2] + c[2], m_t) &&
-                        STATS)
-                        cnt.dropped += m_t;
-                    cnt.add_tgt(P, m_t);
-                    cnt.add_dep(m_t);
-                    if (STATS) {
-                        cnt.u[ts.vol6 == 0.0 ? ST_DEGENERATE : ST_SINGLE_CELL]++;
-                        cnt.u[ST_OVERLAPPED]++;
-                        if (ts.vol6 != 0.0) { cnt.u[ST_BBOX_CELLS]++; cnt.u[ST_BIN0]++; }
+                } else if (flat || ts.vol6 == 0.0 || ncell == 1) {
+                    if (!flat) {
+                        if (ts.vol6 == 0.0) centroid_cell(ts.v, c);
+                        else { c[0] = ts.lo[0]; c[1] = ts.lo[1]; c[2] = ts.lo[2]; }
+                        c[0] += base[0];
+                        c[1] += base[1];
+                        c[2] += base[2];
                     }
-                } else if (int c[3]; !(ts.kappa <= P.kappa_max) && flat_guarded(P, ts, res, base, (int64_t)t, c)) {
                     if (!deposit_cell(P, c[0], c[1], c[2], m_t) && STATS) cnt.dropped += m_t;
                     cnt.add_tgt(P, m_t);
                     cnt.add_dep(m_t);
                     if (STATS) {
-                        cnt.u[ST_DEGENERATE]++;
+                        cnt.u[flat || ts.vol6 == 0.0 ? ST_DEGENERATE : ST_SINGLE_CELL]++;
                         cnt.u[ST_OVERLAPPED]++;
-                        cnt.u[ST_BBOX_CELLS] += ncell;
-                        cnt.u[ST_BIN0 + size_bin(ncell)]++;
+                        if (ts.vol6 != 0.0) { cnt.u[ST_BBOX_CELLS] += ncell; cnt.u[ST_BIN0 + size_bin(ncell)]++; }
                     }
                 } else if (ncell > (int64_t)(1 << 25) || !dims_fit_queue(ts.dim)) {
                     set_error(P.ws, 2, (int)(t & 0x7fffffff));
